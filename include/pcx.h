@@ -464,9 +464,11 @@ pcx_status pcx_precond(pcx_ctx* ctx, const double k[3], double gamma, const void
  * the tensor cores (tcgen05 TF32 with hi/lo error compensation) or the
  * FP32 pipes (register-blocked FMAs, double-float sums across chunks), for
  * na, nb <= 64, even L and 16-byte aligned A, B; a generic CUDA-core
- * kernel otherwise.  PCX_FP64: double-float products and sums on the FP32
- * pipes (error-free product and sum transformations, about 2^-44 relative
- * per term) with the per-block partials summed in FP64.  1 <= na, nb <= 128.
+ * kernel otherwise.  PCX_FP64: 49-bit fixed-point entries below each
+ * column's largest, multiplied exactly as integer digits on the tensor cores
+ * (about 1e-15 of ||A_i|| ||B_j||), per-block partials summed in FP64; a
+ * column with Inf or NaN gives NaN in its row or column of G.
+ * 1 <= na, nb <= 128.
  */
 pcx_status pcx_gram(pcx_ctx* ctx, const void* A, int na, const void* B, int nb, size_t L,
                     int precision, void* G, void* stream);
@@ -491,9 +493,9 @@ int pcx_get_gram_path(void);
  * DEVICE buffer G (G[i*nb + j], interleaved doubles).  The X rows of the
  * Rayleigh-Ritz matrices in the mixed-precision refinement (Sec. 4: LOBPCG
  * with the block X held in FP64 and the search directions in FP32).
- * Accuracy: about 2^-44 relative to ||A_i|| ||B_j|| (double-float sums on
- * the FP32 pipes).  Entries of A must lie inside the FP32 range: magnitudes
- * below 2^-126 count as 0, magnitudes at or above 2^128 give NaN.  A, B, G
+ * Accuracy: about 5e-15 of ||A_i|| ||B_j|| (integer digits on the tensor
+ * cores, as pcx_gram with PCX_FP64).  A column with Inf or NaN gives NaN in
+ * its row or column of G.  A, B, G
  * 16-byte aligned device pointers; 1 <= na, nb <= 128.  Uses a per-device
  * scratch buffer owned by the library: concurrent calls on different streams
  * of one device must be serialised by the caller.

@@ -101,7 +101,7 @@ void pcx_destroy(pcx_ctx* c) {
   for (cudaStream_t st : c->solve_streams) {
     pcx::gram_cc_release_stream(st);
     pcx::gram_tc_release_stream(st);
-    pcx::gram_x_release_stream(st);
+    pcx::gram_digits_release_stream(st);
     pcx::cnn_release_stream(st);
     cudaStreamDestroy(st);
   }
@@ -546,8 +546,8 @@ pcx_status pcx_gram_mixed(pcx_ctx* c, const void* A, int na, const void* B, int 
   if (na < 1 || nb < 1 || na > 128 || nb > 128) return inval(c, "pcx_gram_mixed: need 1 <= na, nb <= 128");
   if (!A || !B || !G || !aligned16(A) || !aligned16(B) || !aligned16(G))
     return inval(c, "pcx_gram_mixed: NULL or misaligned buffer");
-  cudaError_t e = pcx::launch_gram_x(A, na, nullptr, 0, B, nb, L, static_cast<double*>(G),
-                                     static_cast<cudaStream_t>(stream));
+  cudaError_t e = pcx::launch_gram_digits(A, na, B, PCX_FP32, nb, L, static_cast<double*>(G),
+                                          static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? PCX_OK : cuda_fail(c, "pcx_gram_mixed", e);
 }
 

@@ -96,8 +96,7 @@ __global__ void __launch_bounds__(256) gram_kernel(const cx<T>* __restrict__ A, 
 // terms, and accumulated in a double-float pair (Knuth's TwoSum), both
 // error-free transformations of Dekker (1971) and Knuth (TAOCP vol. 2).
 // __fadd_rn / __fmul_rn keep the compiler from fusing the steps.  Entries
-// must stay inside the FP32 exponent range.  (The complex128 Gram products
-// use the same scheme in gram_x.cu.)
+// must stay inside the FP32 exponent range. 
 // ---------------------------------------------------------------------------
 using dfloat::DF;
 
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(256) combine2_kernel(const float4* __restrict_
 
 // ---------------------------------------------------------------------------
 // Combine for complex128 on the FP32 pipes with FP64-level accuracy: the
-// same split / TwoProd / TwoSum scheme as gram_ff_kernel.  Each row's inputs
+// split / TwoProd / TwoSum scheme above.  Each row's inputs
 // are split once and reused for the CY outputs of the sweep; C is split once
 // per CTA into shared memory.
 // ---------------------------------------------------------------------------
@@ -507,7 +506,7 @@ int get_gram_path() { return g_gram_path.load(); }
 
 cudaError_t launch_gram(const void* A, int na, const void* B, int nb, size_t L, int precision, double* G,
                         cudaStream_t s) {
-  if (precision == PCX_FP64) return launch_gram_dd(A, na, B, nb, L, G, s);   // gram_x.cu
+  if (precision == PCX_FP64) return launch_gram_digits(A, na, B, PCX_FP64, nb, L, G, s);
   const int path = g_gram_path.load();
   const bool cc = L > 0 && gram_cc_supported(A, B, na, nb, L);
   const bool tc = L > 0 && gram_tc_supported(na, nb, L);
@@ -515,15 +514,13 @@ cudaError_t launch_gram(const void* A, int na, const void* B, int nb, size_t L, 
     return launch_gram_cc(A, na, B, nb, L, G, s);
   if (tc && path != 2) return launch_gram_tc(A, na, B, nb, L, G, s);
   if (cc) return launch_gram_cc(A, na, B, nb, L, G, s);
-  return launch_gram_cuda_cores(A, na, B, nb, L, precision, G, s);
+  return launch_gram_cuda_cores(A, na, B, nb, L, G, s);
 }
 
-cudaError_t launch_gram_cuda_cores(const void* A, int na, const void* B, int nb, size_t L, int precision, double* G,
-                                   cudaStream_t s) {
+cudaError_t launch_gram_cuda_cores(const void* A, int na, const void* B, int nb, size_t L, double* G, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * 2 * (size_t)na * nb, s);
   if (e != cudaSuccess) return e;
   if (L == 0) return cudaSuccess;
-  if (precision == PCX_FP64) return launch_gram_dd(A, na, B, nb, L, G, s);
   const int tile = GT;
   const int rows_step = GL;
   const unsigned gx = (na + tile - 1) / tile, gy = (nb + tile - 1) / tile;

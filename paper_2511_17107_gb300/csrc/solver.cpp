@@ -33,7 +33,7 @@
 
 // Projection-and-Cholesky-QR passes of the refinement's [P W] block against
 // X.  One: the Rayleigh-Ritz step takes the X-[P W] couplings from exact
-// double-float products of the FP64 X (launch_gram_x), so what FP32
+// digit products of the FP64 X (launch_gram_digits), so what FP32
 // rounding leaves of X in [P W] is accounted for there and a second pass
 // only costs time (measured at 128^3: the same iteration counts, 9% less
 // time per solve).  A build-time choice for tuning builds.
@@ -424,7 +424,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
 // is FP64-accurate; the search directions W = K_P^{-1} R, P and their images
 // are FP32 with FP32 applies.  The Rayleigh-Ritz matrices take their X rows
 // from double-float products of the FP64 X, AX with the FP32 directions
-// (launch_gram_x), their P/W blocks from tensor-core FP32 products, and their
+// (launch_gram_digits), their P/W blocks from tensor-core FP32 products, and their
 // X-X blocks from the previous step (Theta, I).  [P W] is orthonormalised
 // against X in FP32 each step.  An error in a direction block enters the new
 // X scaled by that block's coefficient, which shrinks with the residual, so
@@ -577,7 +577,7 @@ pcx_status lobpcg_refine(Run& r64, Run& r32, int nev, double tol, int maxit, int
     std::vector<cd> gx, grw, gpa, gpb;
     {
       r64.tick(&Times::other);
-      CK(launch_gram_x(r64.S.p, n, nullptr, 0, r32.col(r32.S, n), mp, L, static_cast<double*>(r64.G.p), r64.s));
+      CK(launch_gram_digits(r64.S.p, n, r32.col(r32.S, n), PCX_FP32, mp, L, static_cast<double*>(r64.G.p), r64.s));
       std::vector<cd> gxx((size_t)n * mp);
       CK(cudaMemcpyAsync(gxx.data(), r64.G.p, sizeof(cd) * gxx.size(), cudaMemcpyDeviceToHost, r64.s));
       CK(cudaStreamSynchronize(r64.s));

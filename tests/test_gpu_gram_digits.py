@@ -1,0 +1,122 @@
+"""Digit Gram products (complex128, and complex128 x complex64) against
+extended-precision sums at the edges of the kernel: column counts around the
+tile and launch sizes, row counts around a chunk, columns whose scale rises
+along the rows or differs by hundreds of binary orders, limits of the digits,
+zero columns, Inf and NaN.
+
+Tolerance.  An entry is rounded to 2^-50 2^E with 2^E at most twice the
+column's largest part M; a complex product has two such errors in each of its
+two real terms (2^-46 M M' in all), the digit pairs left out add 2^-45 M M',
+the last group's fraction and its rounding less, so |error| <= L 2^-44 M M'.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _scale(kind, ncol, L, single, rng):
+    lim = 60 if single else 300
+    if kind == "rising":   # grows from row to row: the running exponents change in most chunks
+        return np.tile(2.0 ** np.minimum(np.arange(L) / 11.0, lim), (ncol, 1))
+    if kind == "spread":
+        return np.tile((2.0 ** rng.integers(-lim, lim, size=(ncol, 1))), (1, L))
+    return np.ones((ncol, L))
+
+
+def _block(kind, ncol, L, dtype, seed):
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal((ncol, L)) + 1j * rng.standard_normal((ncol, L))
+    if kind == "limits":   # powers of two, their neighbours below, zeros, subnormals, constant columns
+        eps = np.finfo(np.float32 if dtype == np.complex64 else np.float64).eps
+        tiny = 1e-42 if dtype == np.complex64 else 1e-310
+        vals = np.array([1.0, -1.0, 1 - eps, -(1 - eps / 2), 0.5, 0.0, tiny, 2.0 ** -49, 513 / 1024, -511.5 / 1024])
+        x = rng.choice(vals, size=(ncol, L)) + 1j * rng.choice(vals, size=(ncol, L))
+        x[0] = (1 - eps) * (1 - 1j)
+        x[-1] = 0.0
+    return (x * _scale(kind, ncol, L, dtype == np.complex64, rng)).astype(dtype)
+
+
+def _gram(pcx, a, b):
+    import torch
+    A, B = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    if a is b:
+        B = A
+    G = torch.empty((a.shape[0], b.shape[0]), dtype=torch.complex128, device="cuda")
+    (pcx.pcx_gram if b.dtype == np.complex128 else pcx.pcx_gram_mixed)(A, B, G)
+    return G.cpu().numpy()
+
+
+@pytest.fixture(scope="module")
+def pcx():
+    from paper_2511_17107_gb300 import pcx as p
+    p.lib()
+    return p
+
+
+def _check(a, b, got):
+    L = a.shape[1]
+    want = a.conj().astype(np.clongdouble) @ b.T.astype(np.clongdouble)
+    mag = [np.maximum(np.abs(v.real), np.abs(v.imag)).max(axis=1).astype(np.longdouble) for v in (a, b)]
+    bound = L * np.longdouble(2.0) ** -44 * mag[0][:, None] * mag[1][None, :]
+    assert np.all(np.abs(got - want) <= bound)
+    return want
+
+
+@pytest.mark.parametrize("na,nb", [(1, 1), (7, 9), (8, 8), (16, 32), (17, 23), (33, 40), (48, 48), (49, 12), (5, 97),
+                                   (128, 128)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_shapes(pcx, na, nb, mixed):
+    for L in (1, 31, 33, 700):
+        a = _block("plain", na, L, np.complex128, 1)
+        b = _block("plain", nb, L, np.complex64 if mixed else np.complex128, 2)
+        got = _gram(pcx, a, b)
+        want = _check(a, b, got)
+        norms = np.linalg.norm(a, axis=1)[:, None] * np.linalg.norm(b, axis=1)[None, :]
+        assert np.all(np.abs(got - want) <= 4e-14 * norms)
+
+
+@pytest.mark.parametrize("n", [1, 9, 16, 43, 48, 60])
+def test_hermitian(pcx, n):
+    a = _block("plain", n, 1234, np.complex128, 3)
+    got = _gram(pcx, a, a)
+    _check(a, a, got)
+    if n <= 48:   # one launch: the lower triangle is the exact mirror
+        assert np.array_equal(got, got.conj().T)
+
+
+@pytest.mark.parametrize("kind", ["rising", "spread", "limits"])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_ranges(pcx, kind, mixed):
+    a = _block(kind, 13, 2500, np.complex128, 4)
+    b = _block(kind, 10, 2500, np.complex64 if mixed else np.complex128, 5)
+    _check(a, b, _gram(pcx, a, b))
+    if not mixed:
+        _check(a, a, _gram(pcx, a, a))
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_non_finite(pcx, value):
+    a = _block("plain", 9, 300, np.complex128, 6)
+    b = _block("plain", 6, 300, np.complex64, 7)
+    a[4, 250] = complex(0.0, value)
+    b[2, 3] = complex(value, 1.0)
+    got = _gram(pcx, a, b)
+    bad = np.zeros(got.shape, dtype=bool)
+    bad[4], bad[:, 2] = True, True
+    assert np.all(np.isnan(got[bad].real)) and np.all(np.isnan(got[bad].imag))
+    ra, rb = [i for i in range(9) if i != 4], [j for j in range(6) if j != 2]
+    _check(a[ra], b[rb], got[np.ix_(ra, rb)])
+
+
+def test_long_columns(pcx):
+    """More rows than one CTA takes in a launch of one wave: the exact value of a constant column's Gram."""
+    import torch
+    L = 3 * 10 ** 6
+    A = torch.full((2, L), 1.0 - 2.0 ** -52, dtype=torch.complex128, device="cuda")
+    A[1] = -1j * A[0]
+    G = torch.empty((2, 2), dtype=torch.complex128, device="cuda")
+    pcx.pcx_gram(A, A, G)
+    v = L * (1.0 - 2.0 ** -52) ** 2
+    want = np.array([[v, -1j * v], [1j * v, v]])
+    assert np.abs(G.cpu().numpy() - want).max() <= v * 2.0 ** -44
