@@ -1,5 +1,5 @@
 // complex128 instantiation of the apply and preconditioner kernels.
-#include "fft_kernels.cuh"
+#include "fft_fixed.cuh"
 
 namespace pcx {
 template cudaError_t run_apply_t<double>(const pcx_ctx*, const KParams&, const void*, void*, int, int, void*,

@@ -344,8 +344,142 @@ __device__ __forceinline__ void fft_tile(cx<T>* s, const cx<T>* tw, const cx<T>*
   }
 }
 
+// The kappa tables of an x tile of five-pass geometry (pencils qb ..):
+// kappa_i(p) = sum_j b_ji S_j(p_j) + i kq_i L0(p_i),  S_j = L1 + i kt_j L0,
+// split as ka[i][p1] + kb[t][i] (p2, p3 of pencil t).
+template <typename T, int N>
+__device__ __forceinline__ void pass_kappa_tables(const cx<T>* glam, const KParams& kp, int qb, cx<T>* ka, cx<T>* kb) {
+  using C = Cfg<T, N>;
+  for (int e = threadIdx.x; e < 3 * N + 3 * C::TP; e += C::THREADS) {
+    if (e < 3 * N) {
+      const int i = e / N, p = e % N;
+      const cx<T> l1 = glam[p], l0 = glam[N + p];
+      const T b0 = (T)kp_b(kp, 0, i);   // b_1i (row j = 0)
+      const T kt = (T)kp.kt[0];
+      cx<T> r = mk(b0 * fma(-kt, l0.y, l1.x), b0 * fma(kt, l0.x, l1.y));
+      if (i == 0) r = mk(fma(-(T)kp.kq[0], l0.y, r.x), fma((T)kp.kq[0], l0.x, r.y));
+      ka[e] = r;
+    } else {
+      const int f = e - 3 * N, t = f / 3, i = f % 3;
+      const int q = qb + t, p[3] = {0, q % N, q / N};
+      cx<T> r = mk((T)0, (T)0);
+#pragma unroll
+      for (int j = 1; j < 3; ++j) {
+        const cx<T> l1 = glam[p[j]], l0 = glam[N + p[j]];
+        const T bj = (T)kp_b(kp, j, i), kt = (T)kp.kt[j];
+        r = mk(fma(bj, fma(-kt, l0.y, l1.x), r.x), fma(bj, fma(kt, l0.x, l1.y), r.y));
+        if (i == j) r = mk(fma(-(T)kp.kq[j], l0.y, r.x), fma((T)kp.kq[j], l0.x, r.y));
+      }
+      kb[3 * t + i] = r;
+    }
+  }
+}
+
+// Pass 1 at one mode, kappa_i = ka[i kas] + kb[i]: (x0, x1, x2) becomes u =
+// -conj(kappa) x x and sk = gamma_p kappa.x (T0: u / |k|^2 and kappa.x /
+// (gamma_p |k|^4)).
+template <typename T, bool T0>
+__device__ __forceinline__ void pre_point(cx<T>& x0, cx<T>& x1, cx<T>& x2, cx<T>& sk, const cx<T>* ka, int kas,
+                                          const cx<T>* kb, const KParams& kp, T gam, T igam) {
+  cx<T> kap[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) kap[i] = ka[i * kas] + kb[i];
+  T su = (T)1, ss = gam;
+  if constexpr (T0) {
+    const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
+    su = k2 > (T)0 ? (T)1 / k2 : (T)0;
+    ss = su * su * igam * penalty_inv_weight(kp, k2);
+  } else if (kp.per_mode) {
+    ss = gam * penalty_weight(kp, norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]));
+  }
+  sk = scale(cfma(kap[2], x2, cfma(kap[1], x1, kap[0] * x0)), ss);
+  const cx<T> z = mk((T)0, (T)0);
+  cx<T> u0 = cfma_conj(kap[2], x1, scale(cfma_conj(kap[1], x2, z), (T)-1));
+  cx<T> u1 = cfma_conj(kap[0], x2, scale(cfma_conj(kap[2], x0, z), (T)-1));
+  cx<T> u2 = cfma_conj(kap[1], x0, scale(cfma_conj(kap[0], x1, z), (T)-1));
+  if constexpr (T0) {
+    u0 = scale(u0, su);
+    u1 = scale(u1, su);
+    u2 = scale(u2, su);
+  }
+  x0 = u0;
+  x1 = u1;
+  x2 = u2;
+}
+
+// Pass 5 at one mode: y = C w + conj(kappa) sk (T0: (C w) / |k|^2 + conj(kappa) sk).
+template <typename T, bool T0>
+__device__ __forceinline__ void post_point(const cx<T> w[3], cx<T> sk, const cx<T>* ka, int kas, const cx<T>* kb,
+                                           cx<T>& y0, cx<T>& y1, cx<T>& y2) {
+  cx<T> kap[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) kap[i] = ka[i * kas] + kb[i];
+  cx<T> c0 = cfma(kap[1], w[2], scale(kap[2] * w[1], (T)-1));
+  cx<T> c1 = cfma(kap[2], w[0], scale(kap[0] * w[2], (T)-1));
+  cx<T> c2 = cfma(kap[0], w[1], scale(kap[1] * w[0], (T)-1));
+  if constexpr (T0) {
+    const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
+    const T su = k2 > (T)0 ? (T)1 / k2 : (T)0;
+    c0 = scale(c0, su);
+    c1 = scale(c1, su);
+    c2 = scale(c2, su);
+  }
+  y0 = cfma_conj(kap[0], sk, c0);
+  y1 = cfma_conj(kap[1], sk, c1);
+  y2 = cfma_conj(kap[2], sk, c2);
+}
+
+// e <- s M e in one cell (EPS: s M^{-1} e, M^{-1} = adj(M) / det(M)), the
+// block from the material table (id given) or from the dense blocks M.
+template <typename T, int N, bool EPS>
+__device__ __forceinline__ void cell_point(cx<T> e[3], const uchar4* idp, const T* mtab, const T* M, int cell, T s) {
+  constexpr int N3 = N * N * N;
+  T d1, d2, d3;
+  cx<T> o12, o13, o23;
+  if (idp) {
+    const uchar4 id = *idp;
+    d1 = mtab[9 * id.x];
+    d2 = mtab[9 * id.y + 1];
+    d3 = mtab[9 * id.z + 2];
+    const T* o = mtab + 9 * id.w;
+    o12 = mk(o[3], o[4]);
+    o13 = mk(o[5], o[6]);
+    o23 = mk(o[7], o[8]);
+  } else {
+    d1 = M[cell];
+    d2 = M[N3 + cell];
+    d3 = M[2 * N3 + cell];
+    o12 = mk(M[3 * N3 + cell], M[4 * N3 + cell]);
+    o13 = mk(M[5 * N3 + cell], M[6 * N3 + cell]);
+    o23 = mk(M[7 * N3 + cell], M[8 * N3 + cell]);
+  }
+  if constexpr (EPS) {
+    // the adjugate of the Hermitian block (upper triangle) replaces M, the
+    // determinant joins the scale
+    const T a11 = d2 * d3 - norm2(o23), a22 = d1 * d3 - norm2(o13), a33 = d1 * d2 - norm2(o12);
+    const cx<T> a12 = o13 * conjg(o23) - scale(o12, d3);
+    const cx<T> a13 = o12 * o23 - scale(o13, d2);
+    const cx<T> a23 = o13 * conjg(o12) - scale(o23, d1);
+    const T det = d1 * a11 + (o12 * conjg(a12)).x + (o13 * conjg(a13)).x;
+    s = s / det;
+    d1 = a11;
+    d2 = a22;
+    d3 = a33;
+    o12 = a12;
+    o13 = a13;
+    o23 = a23;
+  }
+  const cx<T> m0 = cfma(o13, e[2], cfma(o12, e[1], scale(e[0], d1)));
+  const cx<T> m1 = cfma(o23, e[2], cfma_conj(o12, e[0], scale(e[1], d2)));
+  const cx<T> m2 = cfma_conj(o23, e[1], cfma_conj(o13, e[0], scale(e[2], d3)));
+  e[0] = scale(m0, s);
+  e[1] = scale(m1, s);
+  e[2] = scale(m2, s);
+}
+
+// complex64 (complex128 passes: pass_fixed_kernel in fft_fixed.cuh)
 template <typename T, int N, int AXIS, int OP>
-__global__ void __launch_bounds__(Cfg<T, N>::THREADS, sizeof(T) == 4 ? 3 : 1) pass_kernel(PassArgs a) {
+__global__ void __launch_bounds__(Cfg<T, N>::THREADS, 3) pass_kernel(PassArgs a) {
   using C = Cfg<T, N>;
   using TL = Tile<T, N, AXIS>;
   constexpr int TP = C::TP;
@@ -367,34 +501,8 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, sizeof(T) == 4 ? 3 : 1) pa
   for (int i = threadIdx.x; i < N; i += C::THREADS) tw[i] = gtw[i];
   KParams kp = a.kp;
   if (AXIS == 0 && a.kps) kp = a.kps[(a.v_base + (int)v) / a.vec_per_k];
-  if constexpr (AXIS == 0 && OP != OP_PLAIN_INV && OP != OP_PLAIN_FWD) {
-    // kappa_i(p) = sum_j b_ji S_j(p_j) + i kq_i L0(p_i),  S_j = L1 + i kt_j L0,
-    // split as ka_i(p1) + kb_i(p2, p3)
-    const cx<T>* glam = static_cast<const cx<T>*>(a.lam);
-    for (int e = threadIdx.x; e < 3 * N + 3 * TP; e += C::THREADS) {
-      if (e < 3 * N) {
-        const int i = e / N, p = e % N;
-        const cx<T> l1 = glam[p], l0 = glam[N + p];
-        const T b0 = (T)kp_b(kp, 0, i);   // b_1i (row j = 0)
-        const T kt = (T)kp.kt[0];
-        cx<T> r = mk(b0 * fma(-kt, l0.y, l1.x), b0 * fma(kt, l0.x, l1.y));
-        if (i == 0) r = mk(fma(-(T)kp.kq[0], l0.y, r.x), fma((T)kp.kq[0], l0.x, r.y));
-        ka[e] = r;
-      } else {
-        const int f = e - 3 * N, t = f / 3, i = f % 3;
-        const int q = qb + t, p[3] = {0, q % N, q / N};
-        cx<T> r = mk((T)0, (T)0);
-#pragma unroll
-        for (int j = 1; j < 3; ++j) {
-          const cx<T> l1 = glam[p[j]], l0 = glam[N + p[j]];
-          const T bj = (T)kp_b(kp, j, i), kt = (T)kp.kt[j];
-          r = mk(fma(bj, fma(-kt, l0.y, l1.x), r.x), fma(bj, fma(kt, l0.x, l1.y), r.y));
-          if (i == j) r = mk(fma(-(T)kp.kq[j], l0.y, r.x), fma((T)kp.kq[j], l0.x, r.y));
-        }
-        kb[3 * t + i] = r;
-      }
-    }
-  }
+  if constexpr (AXIS == 0 && OP != OP_PLAIN_INV && OP != OP_PLAIN_FWD)
+    pass_kappa_tables<T, N>(static_cast<const cx<T>*>(a.lam), kp, qb, ka, kb);
   if constexpr (OP == OP_SANDWICH || OP == OP_SANDWICH_EPS) {
     if (a.mid) {
       const T* gt = static_cast<const T*>(a.mtab);
@@ -427,31 +535,8 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, sizeof(T) == 4 ? 3 : 1) pa
       for (int e = threadIdx.x; e < TP * N; e += C::THREADS) {
         const int t = e / N, n = e % N;
         const int g = TL::gidx(qb + t, n);
-        const cx<T> x0 = s[TL::sidx(0, t, n)], x1 = s[TL::sidx(1, t, n)], x2 = s[TL::sidx(2, t, n)];
-        cx<T> kap[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) kap[i] = ka[i * N + n] + kb[3 * t + i];
-        T su = (T)1, ss = gam;
-        if constexpr (OP == OP_PRE_T0) {
-          const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
-          su = k2 > (T)0 ? (T)1 / k2 : (T)0;
-          ss = su * su * igam * penalty_inv_weight(kp, k2);
-        } else if (kp.per_mode) {
-          ss = gam * penalty_weight(kp, norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]));
-        }
-        sb[g] = scale(cfma(kap[2], x2, cfma(kap[1], x1, kap[0] * x0)), ss);
-        const cx<T> z = mk((T)0, (T)0);
-        cx<T> u0 = cfma_conj(kap[2], x1, scale(cfma_conj(kap[1], x2, z), (T)-1));
-        cx<T> u1 = cfma_conj(kap[0], x2, scale(cfma_conj(kap[2], x0, z), (T)-1));
-        cx<T> u2 = cfma_conj(kap[1], x0, scale(cfma_conj(kap[0], x1, z), (T)-1));
-        if constexpr (OP == OP_PRE_T0) {
-          u0 = scale(u0, su);
-          u1 = scale(u1, su);
-          u2 = scale(u2, su);
-        }
-        s[TL::sidx(0, t, n)] = u0;
-        s[TL::sidx(1, t, n)] = u1;
-        s[TL::sidx(2, t, n)] = u2;
+        pre_point<T, OP == OP_PRE_T0>(s[TL::sidx(0, t, n)], s[TL::sidx(1, t, n)], s[TL::sidx(2, t, n)], sb[g], ka + n, N,
+                                      kb + 3 * t, kp, gam, igam);
       }
       __syncthreads();
       fft_tile<T, N, 0, +1, 0, 1>(s, tw, nullptr, out, qb);
@@ -470,24 +555,8 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, sizeof(T) == 4 ? 3 : 1) pa
       for (int e = threadIdx.x; e < TP * N; e += C::THREADS) {
         const int t = e / N, n = e % N;
         const int g = TL::gidx(qb + t, n);
-        const cx<T> sk = ssb[e];
-        cx<T> kap[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) kap[i] = ka[i * N + n] + kb[3 * t + i];
-        const cx<T> w0 = s[TL::sidx(0, t, n)], w1 = s[TL::sidx(1, t, n)], w2 = s[TL::sidx(2, t, n)];
-        cx<T> c0 = cfma(kap[1], w2, scale(kap[2] * w1, (T)-1));
-        cx<T> c1 = cfma(kap[2], w0, scale(kap[0] * w2, (T)-1));
-        cx<T> c2 = cfma(kap[0], w1, scale(kap[1] * w0, (T)-1));
-        if constexpr (OP == OP_POST_T0) {
-          const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
-          const T su = k2 > (T)0 ? (T)1 / k2 : (T)0;
-          c0 = scale(c0, su);
-          c1 = scale(c1, su);
-          c2 = scale(c2, su);
-        }
-        out[g] = cfma_conj(kap[0], sk, c0);
-        out[N3 + g] = cfma_conj(kap[1], sk, c1);
-        out[2 * N3 + g] = cfma_conj(kap[2], sk, c2);
+        const cx<T> w[3] = {s[TL::sidx(0, t, n)], s[TL::sidx(1, t, n)], s[TL::sidx(2, t, n)]};
+        post_point<T, OP == OP_POST_T0>(w, ssb[e], ka + n, N, kb + 3 * t, out[g], out[N3 + g], out[2 * N3 + g]);
       }
     }
   } else if constexpr (OP == OP_SANDWICH || OP == OP_SANDWICH_EPS) {
@@ -512,51 +581,11 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, sizeof(T) == 4 ? 3 : 1) pa
     const T inv_n3 = (T)(1.0 / (double)N3);
     for (int w = threadIdx.x; w < TP * N; w += C::THREADS) {   // pencils fastest
       const int t = w % TP, n = w / TP;
-      const int cell = n * N2 + (qb + t);   // (x, y, z) = (q % N, q / N, n)
-      T d1, d2, d3;
-      cx<T> o12, o13, o23;
-      if (mid) {
-        const uchar4 id = sid[w];
-        d1 = mtab[9 * id.x];
-        d2 = mtab[9 * id.y + 1];
-        d3 = mtab[9 * id.z + 2];
-        const T* o = mtab + 9 * id.w;
-        o12 = mk(o[3], o[4]);
-        o13 = mk(o[5], o[6]);
-        o23 = mk(o[7], o[8]);
-      } else {
-        d1 = M[cell];
-        d2 = M[N3 + cell];
-        d3 = M[2 * N3 + cell];
-        o12 = mk(M[3 * N3 + cell], M[4 * N3 + cell]);
-        o13 = mk(M[5 * N3 + cell], M[6 * N3 + cell]);
-        o23 = mk(M[7 * N3 + cell], M[8 * N3 + cell]);
-      }
-      const int i0 = TL::sidx(0, t, n), i1 = TL::sidx(1, t, n), i2 = TL::sidx(2, t, n);
-      const cx<T> e0 = s[i0], e1 = s[i1], e2 = s[i2];
-      T sc = inv_n3;
-      if constexpr (OP == OP_SANDWICH_EPS) {
-        // eps = M^{-1} = adj(M) / det(M): the adjugate of the Hermitian block
-        // (upper triangle) replaces M, the determinant joins the scale
-        const T a11 = d2 * d3 - norm2(o23), a22 = d1 * d3 - norm2(o13), a33 = d1 * d2 - norm2(o12);
-        const cx<T> a12 = o13 * conjg(o23) - scale(o12, d3);
-        const cx<T> a13 = o12 * o23 - scale(o13, d2);
-        const cx<T> a23 = o13 * conjg(o12) - scale(o23, d1);
-        const T det = d1 * a11 + (o12 * conjg(a12)).x + (o13 * conjg(a13)).x;
-        sc = inv_n3 / det;
-        d1 = a11;
-        d2 = a22;
-        d3 = a33;
-        o12 = a12;
-        o13 = a13;
-        o23 = a23;
-      }
-      const cx<T> m0 = cfma(o13, e2, cfma(o12, e1, scale(e0, d1)));
-      const cx<T> m1 = cfma(o23, e2, cfma_conj(o12, e0, scale(e1, d2)));
-      const cx<T> m2 = cfma_conj(o23, e1, cfma_conj(o13, e0, scale(e2, d3)));
-      s[i0] = scale(m0, sc);
-      s[i1] = scale(m1, sc);
-      s[i2] = scale(m2, sc);
+      // cell (x, y, z) = (q % N, q / N, n), q = qb + t
+      cx<T> e[3] = {s[TL::sidx(0, t, n)], s[TL::sidx(1, t, n)], s[TL::sidx(2, t, n)]};
+      cell_point<T, N, OP == OP_SANDWICH_EPS>(e, mid ? &sid[w] : nullptr, mtab, M, n * N2 + (qb + t), inv_n3);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) s[TL::sidx(c, t, n)] = e[c];
     }
     __syncthreads();
     fft_tile<T, N, 2, -1, 0, 1>(s, tw, nullptr, out, qb);
@@ -862,9 +891,20 @@ __global__ void crossdof_kernel(const cx<T>* __restrict__ E, cx<T>* __restrict__
   }
 }
 
+// complex128: the pass with its transforms in fixed point (fft_fixed.cuh)
+namespace fixed {
+template <int N, int AXIS, int OP>
+__global__ void pass_fixed_kernel(PassArgs a);
+}
+template <typename T, int N, int AXIS, int OP>
+constexpr auto pass_entry() {
+  if constexpr (sizeof(T) == 8) return fixed::pass_fixed_kernel<N, AXIS, OP>;
+  else return pass_kernel<T, N, AXIS, OP>;
+}
+
 template <typename T, int N, int AXIS, int OP>
 cudaError_t launch_pass(const PassArgs& a, size_t tiles, size_t smem, cudaStream_t st) {
-  auto kern = pass_kernel<T, N, AXIS, OP>;
+  const auto kern = pass_entry<T, N, AXIS, OP>();
   cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)tiles, Cfg<T, N>::THREADS, smem, st>>>(a);
