@@ -56,8 +56,8 @@ cudaError_t adjoint_weights(const float* w, int cout, int cin, float* wt, cudaSt
 // dz = (sum_b dh[b] a[b]) g (1 - g);  dh[b] <- dh[b] g   (gate backward)
 cudaError_t gate_backward(const View& dh, const View& a, const float* g, int nb, int c, size_t n3, float* dz,
                           cudaStream_t s);
-// db[ch] (+)= sum_v dz[ch][v]
-cudaError_t bias_grad(const float* dz, int c, size_t n3, float* db, int accumulate, cudaStream_t s);
+// db[ch] (+)= sum_v dz[ch][v], c <= 32; scratch: 32 doubles per channel
+cudaError_t bias_grad(const float* dz, int c, size_t n3, float* db, int accumulate, float* scratch, cudaStream_t s);
 // dY = 2 w_v (Y - T) over complex64 blocks; loss[0] += sum_v w_v ||Y_v - T_v||^2
 cudaError_t loss_grad(const void* Y, const void* T, const double* wv, int nvec, size_t n3, void* dY, double* loss,
                       cudaStream_t s);

@@ -265,9 +265,9 @@ cudaError_t cnn_grad(pcx_ctx* c, const float* params, const void* U, const void*
   }
   // gate parameters
   CKE(cnn::conv_wgrad(9, C, cnn::dense_view(dz1, C, n3), fv, 1, n, grad + cnn::OFF_V1, accumulate, scr, s));
-  CKE(cnn::bias_grad(dz1, C, n3, grad + cnn::OFF_C1, accumulate, s));
+  CKE(cnn::bias_grad(dz1, C, n3, grad + cnn::OFF_C1, accumulate, scr, s));
   CKE(cnn::conv_wgrad(9, C, cnn::dense_view(dz2, C, n3), fv, 1, n, grad + cnn::OFF_V2, accumulate, scr, s));
-  CKE(cnn::bias_grad(dz2, C, n3, grad + cnn::OFF_C2, accumulate, s));
+  CKE(cnn::bias_grad(dz2, C, n3, grad + cnn::OFF_C2, accumulate, scr, s));
   if (loss_host) {
     CKE(cudaMemcpyAsync(loss_host, ldev, sizeof(double), cudaMemcpyDeviceToHost, s));
     CKE(cudaStreamSynchronize(s));
