@@ -204,10 +204,11 @@ pcx_status pcx_symbols(const pcx_ctx* ctx, const double k[3], double gamma,
                        double* s_tab, double* q_tab, double* b, double* gamma_out);
 
 /*
- * pcx_set_apply_chunk -- tuning knob of pcx_apply: the number of vectors
- * that run through all five FFT passes before the next ones start (their
- * work space is meant to stay resident in L2).  chunk <= 0 restores the
- * default (largest count whose vectors fill at most half of L2, >= 1).
+ * pcx_set_apply_chunk -- tuning knob of pcx_apply: the largest number of
+ * vectors that run through all FFT passes before the next ones start (a block
+ * is split into launches of equal size).  chunk <= 0 restores the default:
+ * as many vectors as 256 MiB of scratch hold (one at least), or for
+ * M_CrossDoF a single vector where half of L2 holds no more.
  * Host-only; affects calls issued afterwards.
  */
 pcx_status pcx_set_apply_chunk(pcx_ctx* ctx, int chunk);

@@ -48,12 +48,25 @@ cudaError_t dispatch_apply(const pcx_ctx* c, const KParams& kp, const void* X, v
 }
 }  // namespace
 
+// Default chunk.  The passes are not bound by DRAM (a vector costs the same
+// with its intermediates in L2 or not), while a launch of few tiles loses its
+// last wave and its ramp: at 128^3 in complex64 one vector per launch takes
+// 109.7 us, 16 take 99.1 us each; at 64^3, 13 vectors in one launch 13.9 us
+// each, 10 and 3 14.7 us; in complex128 at 128^3 836 against 774 us.  So a
+// chunk is as many vectors as a scratch of 256 MiB holds.  The M_CrossDoF
+// chain keeps one vector per launch where that is what half of L2 holds (its
+// stencil pass reads every value 9 times: 173 us at 128^3 against 177), and a
+// context whose scratch could not be allocated stays with what half of L2
+// holds.
 int apply_chunk(const pcx_ctx* c, int precision) {
   if (c->apply_chunk > 0) return c->apply_chunk;
-  const size_t vbytes = (size_t)3 * c->n * c->n * c->n * (precision == PCX_FP64 ? 16 : 8);
+  const size_t es = precision == PCX_FP64 ? 16 : 8, n3 = (size_t)c->n * c->n * c->n;
   const size_t l2 = c->l2_bytes ? c->l2_bytes : ((size_t)126 << 20);
-  const size_t k = (l2 / 2) / vbytes;
-  return (int)(k < 1 ? 1 : (k > 64 ? 64 : k));
+  const size_t k = (l2 / 2) / (3 * n3 * es);
+  const bool cross = c->m_kind == PCX_M_CROSSDOF;
+  if (c->small_scratch || (cross && k <= 1)) return (int)(k < 1 ? 1 : (k > 64 ? 64 : k));
+  const size_t fit = ((size_t)256 << 20) / (n3 * es * (cross ? 4 : 1));
+  return (int)(fit < 1 ? 1 : (fit > 4096 ? 4096 : fit));
 }
 
 cudaError_t raise_dyn_smem(const void* func, size_t bytes) {
@@ -144,7 +157,7 @@ cudaError_t launch_apply_noalloc(const pcx_ctx* c, const KParams& kp, const void
 namespace {
 
 cudaError_t ensure_scratch(pcx_ctx* c, int precision, int nvec) {
-  const size_t need = apply_scratch_bytes(c, precision, nvec);
+  size_t need = apply_scratch_bytes(c, precision, nvec);
   if (need > c->scratch_bytes) {
     // the previous scratch may still be in use by work queued on another stream
     cudaError_t e = cudaDeviceSynchronize();
@@ -154,6 +167,12 @@ cudaError_t ensure_scratch(pcx_ctx* c, int precision, int nvec) {
     c->scratch = nullptr;
     c->scratch_bytes = 0;
     e = cudaMalloc(&c->scratch, need);
+    if (e == cudaErrorMemoryAllocation && !c->small_scratch) {   // smaller chunks from now on
+      cudaGetLastError();
+      c->small_scratch = 1;
+      need = apply_scratch_bytes(c, precision, nvec);
+      e = cudaMalloc(&c->scratch, need);
+    }
     if (e != cudaSuccess) return e;
     c->scratch_bytes = need;
   }

@@ -948,6 +948,10 @@ cudaError_t run_apply_n(const pcx_ctx* c, const KParams& kp, const void* X, void
   // forward z transform
   const bool crossdof = c->m_kind == PCX_M_CROSSDOF && !t0;
   const int cap = nvec < chunk ? nvec : chunk;   // vectors the scratch holds
+  if (nvec > chunk) {   // launches of equal size (13 vectors, chunk 10: 7 and 6)
+    const int parts = (nvec + chunk - 1) / chunk;
+    chunk = (nvec + parts - 1) / parts;
+  }
   cx<T>* tmp = static_cast<cx<T>*>(sbuf) + (size_t)cap * N * N * N;
   for (int v0 = 0; v0 < nvec; v0 += chunk) {
     const int nv = nvec - v0 < chunk ? nvec - v0 : chunk;

@@ -72,8 +72,9 @@ struct pcx_ctx {
   std::vector<double> blocks;            // host N^3 x 9 packed cell blocks
   double lambda_min = 0.0;
   pcx::DeviceTables dev;
-  // apply tuning and scratch: vectors per L2-resident chunk (0 = from L2 size)
+  // apply tuning and scratch: vectors per launch chunk (0 = the default of apply_chunk())
   int apply_chunk = 0;
+  int small_scratch = 0;   // 1 after a scratch allocation failed: default chunks from L2 size
   // apply pass structure: PCX_APPLY_AUTO, PCX_APPLY_FIVE_PASS or PCX_APPLY_THREE_PASS
   int apply_path = 0;
   // kernel variants of the three-pass chain's x and z passes (-1: build default)

@@ -880,8 +880,23 @@ pcx_status solve_concurrent(KSolve& base, const double* kpts, int nk, double pen
     return PCX_ECUDA;
   }
   // apply / T0 scratch of one slot: the larger of the two precisions' needs
+  // (allocated here, before the slots start; smaller chunks where it does not fit)
   const int n3cols = 3 * base.n;
-  const size_t scr = std::max(apply_scratch_bytes(c, PCX_FP64, n3cols), apply_scratch_bytes(c, PCX_FP32, n3cols));
+  std::vector<DevBuf> ascrs(conc);
+  for (;;) {
+    const size_t scr = std::max(apply_scratch_bytes(c, PCX_FP64, n3cols), apply_scratch_bytes(c, PCX_FP32, n3cols));
+    e = cudaSuccess;
+    for (int w = 0; w < conc && e == cudaSuccess; ++w) e = ascrs[w].alloc(scr);
+    if (e != cudaErrorMemoryAllocation || c->small_scratch) break;
+    cudaGetLastError();
+    c->small_scratch = 1;
+    ascrs = std::vector<DevBuf>(conc);
+  }
+  if (e != cudaSuccess) {
+    cudaEventDestroy(ready);
+    c->err = std::string("pcx_solve: ") + cudaGetErrorString(e);
+    return e == cudaErrorMemoryAllocation ? PCX_ENOMEM : PCX_ECUDA;
+  }
   std::atomic<int> next{0};
   std::atomic<bool> failed{false};
   std::mutex mu;
@@ -919,16 +934,13 @@ pcx_status solve_concurrent(KSolve& base, const double* kpts, int nk, double pen
     };
     cudaError_t ee = cudaSetDevice(c->device);
     if (ee == cudaSuccess) ee = cudaStreamWaitEvent(sl.ks.s, ready, 0);
-    DevBuf ascr;
-    if (ee == cudaSuccess) ee = ascr.alloc(scr);
     if (ee != cudaSuccess) {
-      fail(ee == cudaErrorMemoryAllocation ? PCX_ENOMEM : PCX_ECUDA,
-           std::string("pcx_solve: ") + cudaGetErrorString(ee));
+      fail(PCX_ECUDA, std::string("pcx_solve: ") + cudaGetErrorString(ee));
       return;
     }
     Run r64, r32;
-    r64.ascr = ascr.p;
-    r32.ascr = ascr.p;
+    r64.ascr = ascrs[w].p;
+    r32.ascr = ascrs[w].p;
     for (int ik = next++; ik < nk && !failed; ik = next++) {
       bool noconv = false;
       pcx_status st = solve_k(sl.ks, kpts + 3 * ik, ik, penalty_tol, out, r64, r32, sl.raises, sl.gamma_last, noconv);
