@@ -34,6 +34,7 @@
 #include <cstdint>
 
 #include "cnn.h"
+#include "cx.cuh"
 #include "pcx_internal.h"
 
 namespace pcx {
@@ -109,13 +110,6 @@ __device__ __forceinline__ void load_halo(float* sx, const View& in, int b, int 
 #pragma unroll
     for (int i = 0; i < TS; ++i) d[1 + i] = v[i];
   }
-}
-
-// d += a b on two floats (one instruction; each as fmaf)
-__device__ __forceinline__ void fma2(float2& d, float2 a, float2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;\n"
-      : "+l"(reinterpret_cast<unsigned long long&>(d))
-      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
 }
 
 // out[b][co] = conv(in[b], w)[co]            (MODE_PLAIN), times out_scale

@@ -45,6 +45,13 @@ __device__ __forceinline__ cx<T> cfma_conj(cx<T> b, cx<T> c, cx<T> a) {
 template <typename T>
 __device__ __forceinline__ T norm2(cx<T> a) { return fma(a.x, a.x, a.y * a.y); }
 
+// d += a b on two floats, one instruction (each as fmaf)
+__device__ __forceinline__ void fma2(float2& d, float2 a, float2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;\n"
+      : "+l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+}
+
 // cos and sin of 2 pi m / 16, m = 0..15 (numeric values of the circle points).
 __host__ __device__ constexpr double cos16(int m) {
   return m == 0 ? 1.0 : m == 1 ? 0.92387953251128675613 : m == 2 ? 0.70710678118654752440
