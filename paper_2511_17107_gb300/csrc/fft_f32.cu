@@ -1,5 +1,6 @@
 // complex64 instantiation of the apply and preconditioner kernels.
 #include "fft3_kernels.cuh"
+#include "fft_small.cuh"
 
 namespace pcx {
 template cudaError_t run_apply_t<float>(const pcx_ctx*, const KParams&, const void*, void*, int, int, void*,

@@ -344,13 +344,12 @@ __device__ __forceinline__ void fft_tile(cx<T>* s, const cx<T>* tw, const cx<T>*
   }
 }
 
-// The kappa tables of an x tile of five-pass geometry (pencils qb ..):
-// kappa_i(p) = sum_j b_ji S_j(p_j) + i kq_i L0(p_i),  S_j = L1 + i kt_j L0,
-// split as ka[i][p1] + kb[t][i] (p2, p3 of pencil t).
-template <typename T, int N>
-__device__ __forceinline__ void pass_kappa_tables(const cx<T>* glam, const KParams& kp, int qb, cx<T>* ka, cx<T>* kb) {
-  using C = Cfg<T, N>;
-  for (int e = threadIdx.x; e < 3 * N + 3 * C::TP; e += C::THREADS) {
+// The kappa tables of TP x pencils q = qb ..: kappa_i(p) = sum_j b_ji
+// S_j(p_j) + i kq_i L0(p_i),  S_j = L1 + i kt_j L0, split as ka[i][p1] +
+// kb[t][i] (p2, p3 of pencil t).
+template <typename T, int N, int TP, int THREADS>
+__device__ __forceinline__ void kappa_tables(const cx<T>* glam, const KParams& kp, int qb, cx<T>* ka, cx<T>* kb) {
+  for (int e = threadIdx.x; e < 3 * N + 3 * TP; e += THREADS) {
     if (e < 3 * N) {
       const int i = e / N, p = e % N;
       const cx<T> l1 = glam[p], l0 = glam[N + p];
@@ -373,6 +372,11 @@ __device__ __forceinline__ void pass_kappa_tables(const cx<T>* glam, const KPara
       kb[3 * t + i] = r;
     }
   }
+}
+// the same for a tile of the five passes
+template <typename T, int N>
+__device__ __forceinline__ void pass_kappa_tables(const cx<T>* glam, const KParams& kp, int qb, cx<T>* ka, cx<T>* kb) {
+  kappa_tables<T, N, Cfg<T, N>::TP, Cfg<T, N>::THREADS>(glam, kp, qb, ka, kb);
 }
 
 // Pass 1 at one mode, kappa_i = ka[i kas] + kb[i]: (x0, x1, x2) becomes u =
@@ -911,6 +915,15 @@ __host__ __device__ constexpr bool has_pass3() {
 template <typename T, int N, int OP>
 cudaError_t launch_pass3(const PassArgs& a, int nv, cudaStream_t st, int xv, int zv);
 
+// The five passes of a vector in one launch (fft_small.cuh): complex64 at
+// N = 8, 16, where a vector fits an SM's shared memory.
+template <typename T, int N>
+__host__ __device__ constexpr bool has_small() {
+  return sizeof(T) == 4 && N <= 16;
+}
+template <typename T, int N, bool T0>
+cudaError_t launch_small(const PassArgs& a, int nv, cudaStream_t st);
+
 template <typename T, int N>
 cudaError_t run_apply_n(const pcx_ctx* c, const KParams& kp, const void* X, void* Y, int nvec, int chunk, void* sbuf,
                         cudaStream_t st, const KParams* kps, int vec_per_k, bool t0) {
@@ -977,36 +990,40 @@ cudaError_t run_apply_n(const pcx_ctx* c, const KParams& kp, const void* X, void
     }
     a.in = x;
     a.out = y;
-    if constexpr (has_pass3<T, N>()) {
-      if (c->apply_path != PCX_APPLY_FIVE_PASS && (c->dev.mid3 || !c->dev.mid)) {
-        // three passes, in place on y after the first
-        a.mid3 = c->dev.mid3;
-        const int xv = c->x3_variant, zv = c->z3_variant;
-        if ((e = t0 ? launch_pass3<T, N, OP_PRE_T0>(a, nv, st, xv, zv) : launch_pass3<T, N, OP_PRE>(a, nv, st, xv, zv))
-            != cudaSuccess)
-          return e;
-        a.in = y;
-        if ((e = t0 ? launch_pass3<T, N, OP_SANDWICH_EPS>(a, nv, st, xv, zv)
-                    : launch_pass3<T, N, OP_SANDWICH>(a, nv, st, xv, zv)) != cudaSuccess)
-          return e;
-        if ((e = t0 ? launch_pass3<T, N, OP_POST_T0>(a, nv, st, xv, zv) : launch_pass3<T, N, OP_POST>(a, nv, st, xv, zv))
-            != cudaSuccess)
-          return e;
-        continue;
+    if constexpr (has_small<T, N>()) {
+      if ((e = t0 ? launch_small<T, N, true>(a, nv, st) : launch_small<T, N, false>(a, nv, st)) != cudaSuccess) return e;
+    } else {
+      if constexpr (has_pass3<T, N>()) {
+        if (c->apply_path != PCX_APPLY_FIVE_PASS && (c->dev.mid3 || !c->dev.mid)) {
+          // three passes, in place on y after the first
+          a.mid3 = c->dev.mid3;
+          const int xv = c->x3_variant, zv = c->z3_variant;
+          if ((e = t0 ? launch_pass3<T, N, OP_PRE_T0>(a, nv, st, xv, zv) : launch_pass3<T, N, OP_PRE>(a, nv, st, xv, zv))
+              != cudaSuccess)
+            return e;
+          a.in = y;
+          if ((e = t0 ? launch_pass3<T, N, OP_SANDWICH_EPS>(a, nv, st, xv, zv)
+                      : launch_pass3<T, N, OP_SANDWICH>(a, nv, st, xv, zv)) != cudaSuccess)
+            return e;
+          if ((e = t0 ? launch_pass3<T, N, OP_POST_T0>(a, nv, st, xv, zv) : launch_pass3<T, N, OP_POST>(a, nv, st, xv, zv))
+              != cudaSuccess)
+            return e;
+          continue;
+        }
       }
+      if ((e = t0 ? launch_pass<T, N, 0, OP_PRE_T0>(a, tiles, smem, st) : launch_pass<T, N, 0, OP_PRE>(a, tiles, smem, st))
+          != cudaSuccess)
+        return e;
+      a.in = y;
+      if ((e = launch_pass<T, N, 1, OP_INV>(a, tiles, smem, st)) != cudaSuccess) return e;
+      if ((e = t0 ? launch_pass<T, N, 2, OP_SANDWICH_EPS>(a, tiles, sandwich_smem, st)
+                  : launch_pass<T, N, 2, OP_SANDWICH>(a, tiles, sandwich_smem, st)) != cudaSuccess)
+        return e;
+      if ((e = launch_pass<T, N, 1, OP_FWD>(a, tiles, smem, st)) != cudaSuccess) return e;
+      if ((e = t0 ? launch_pass<T, N, 0, OP_POST_T0>(a, tiles, post_smem, st)
+                  : launch_pass<T, N, 0, OP_POST>(a, tiles, post_smem, st)) != cudaSuccess)
+        return e;
     }
-    if ((e = t0 ? launch_pass<T, N, 0, OP_PRE_T0>(a, tiles, smem, st) : launch_pass<T, N, 0, OP_PRE>(a, tiles, smem, st))
-        != cudaSuccess)
-      return e;
-    a.in = y;
-    if ((e = launch_pass<T, N, 1, OP_INV>(a, tiles, smem, st)) != cudaSuccess) return e;
-    if ((e = t0 ? launch_pass<T, N, 2, OP_SANDWICH_EPS>(a, tiles, sandwich_smem, st)
-                : launch_pass<T, N, 2, OP_SANDWICH>(a, tiles, sandwich_smem, st)) != cudaSuccess)
-      return e;
-    if ((e = launch_pass<T, N, 1, OP_FWD>(a, tiles, smem, st)) != cudaSuccess) return e;
-    if ((e = t0 ? launch_pass<T, N, 0, OP_POST_T0>(a, tiles, post_smem, st)
-                : launch_pass<T, N, 0, OP_POST>(a, tiles, post_smem, st)) != cudaSuccess)
-      return e;
   }
   return cudaSuccess;
 }
