@@ -374,7 +374,8 @@ int pcx_get_penalty_form(const pcx_ctx* ctx);
  *   z_variant (pass B): 0 -- one z tile per CTA; 1 -- a persistent
  *     warp-specialised kernel, one CTA per SM, in which half the warps
  *     transform one tile buffer while the other half store the previous
- *     tile and load the next one into the second buffer.
+ *     tile and load the next one into the second buffer (N = 32 and 64; at
+ *     N = 128, where one tile fills an SM, it runs as 0).
  * -1 selects the build's default (x 3, z 0).  pcx_autotune sets both.
  * Changing them frees the captured apply graphs.  PCX_EINVAL out of range.
  */

@@ -43,29 +43,36 @@ namespace fftk {
 template <int N>
 struct YSplit;
 template <> struct YSplit<32> { static constexpr int RA = 8, RB = 4; };
-template <> struct YSplit<64> { static constexpr int RA = 8, RB = 8; };
+template <> struct YSplit<64> { static constexpr int RA = 16, RB = 4; };
 template <> struct YSplit<128> { static constexpr int RA = 16, RB = 8; };
 
-// Geometry of the z tiles (pass B): RB rows x TPX columns of z pencils, at
-// least 32 bytes of consecutive x per row so that every global access of
-// the pass fills whole 32-byte sectors.  At N = 128 that is 32 pencils
-// (96 KB of complex64 for the three components), two CTAs per SM of 256
-// threads with 48 elements per thread and stage: the fused inverse-stage /
-// M / forward-stage step holds three components of eight points, which
-// needs more than the 80 registers a 384-thread CTA could have.
+// Geometry of the z tiles (pass B): RB rows x TPX columns of z pencils.  A
+// global access of the pass reads or writes TPX consecutive entries of a row,
+// and short pieces cost more than the lost overlap of smaller tiles: 64 bytes
+// (N = 128) or 128 (N = 64, 32) measured fastest.  Per 16 (N = 128) and 13 or
+// 48 (N = 64) complex64 vectors, us, apply / T0:
+//   N = 128, 32-byte pieces, two CTAs of 256 threads   1599 / 1805
+//   N = 128, 64-byte pieces, one CTA of 512            1571 / 1703
+//   N = 64 = 8 x 8, 32-byte, two CTAs of 384            181 / 197,  619 / 671
+//   N = 64 = 8 x 8, 64-byte, two CTAs of 256            165 / 179,  552 / 608
+//   N = 64 = 16 x 4, 128-byte, two CTAs of 256          156 / 167,  528 / 574
+// The threads hold 48 elements per stage: the fused inverse-stage / M /
+// forward-stage step keeps three components of eight points in registers
+// (about 128 of them), more than a CTA of 24 warps could have.
 #ifndef PCX_Z128_TN
-#define PCX_Z128_TN 4096
+#define PCX_Z128_TN 8192
 #endif
 #ifndef PCX_Z128_E
 #define PCX_Z128_E 48
 #endif
 #ifndef PCX_Z128_MINB
-#define PCX_Z128_MINB 2
+#define PCX_Z128_MINB 1
 #endif
 template <int N>
 struct ZGeom {
   static constexpr int TN = 2048, E = 16, MINB = 2;
 };
+template <> struct ZGeom<64> { static constexpr int TN = 4096, E = 48, MINB = 2; };
 template <> struct ZGeom<128> { static constexpr int TN = PCX_Z128_TN, E = PCX_Z128_E, MINB = PCX_Z128_MINB; };
 
 // Row padding of the z tiles.  Pass B's y DFTs stage two x columns per
@@ -867,6 +874,12 @@ __global__ void pass3_ids_kernel(const uchar4* __restrict__ mid, uchar4* __restr
   }
 }
 
+// shared copy of the material table (none where pass B reads it through L1)
+template <typename T, int N, int OP>
+size_t mtab_smem(int n_mat) {
+  return ZTile<T, N, OP>::GTAB ? 0 : (((size_t)12 * n_mat * sizeof(T) + 15) & ~(size_t)15);
+}
+
 // One pass of the three-pass chain over nv vectors; the shared memory of
 // each tile kind is fixed by its geometry (x tiles: the five-pass x layout
 // plus the kappa tables; z tiles: the tile, the twiddles and the material
@@ -877,7 +890,7 @@ cudaError_t launch_pass3_tile(const PassArgs& a, int nv, cudaStream_t st) {
   constexpr bool ZP = is_z_op<OP>();
   size_t smem;
   if constexpr (ZP)
-    smem = C3::ZSMEM_TILE + (size_t)N * sizeof(cx<T>) + (((size_t)12 * a.n_mat * sizeof(T) + 15) & ~(size_t)15);
+    smem = C3::ZSMEM_TILE + (size_t)N * sizeof(cx<T>) + mtab_smem<T, N, OP>(a.n_mat);
   else
     smem = C3::C::SMEM;
   const size_t tiles = (size_t)nv * (ZP ? C3::ZTILES : C3::TILES);
@@ -891,8 +904,7 @@ cudaError_t launch_pass3_tile(const PassArgs& a, int nv, cudaStream_t st) {
 template <typename T, int N, int OP>
 cudaError_t launch_pass3_ws(const PassArgs& a, int nv, cudaStream_t st) {
   using C3 = Cfg3<T, N>;
-  const size_t smem = 2 * C3::ZSMEM_TILE + (size_t)N * sizeof(cx<T>) +
-                      (((size_t)12 * a.n_mat * sizeof(T) + 15) & ~(size_t)15);
+  const size_t smem = 2 * C3::ZSMEM_TILE + (size_t)N * sizeof(cx<T>) + mtab_smem<T, N, OP>(a.n_mat);
   const long long tiles = (long long)nv * C3::ZTILES;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
@@ -944,7 +956,12 @@ template <typename T, int N, int OP>
 cudaError_t launch_pass3(const PassArgs& a, int nv, cudaStream_t st, int xv, int zv) {
   if constexpr (is_z_op<OP>()) {
     if (zv < 0 || zv >= Z3_VARIANTS) zv = PCX_Z3_VARIANT;
-    return zv == 1 ? launch_pass3_ws<T, N, OP>(a, nv, st) : launch_pass3_tile<T, N, OP, 0>(a, nv, st);
+    // two tile buffers must fit an SM for the warp-specialised kernel; the
+    // 128-point tiles, of which one fills it, take the other kernel
+    if constexpr (2 * Cfg3<T, N>::ZSMEM_TILE + N * sizeof(cx<T>) <= (size_t)227 * 1024) {
+      if (zv == 1) return launch_pass3_ws<T, N, OP>(a, nv, st);
+    }
+    return launch_pass3_tile<T, N, OP, 0>(a, nv, st);
   } else {
     if (xv < 0 || xv >= X3_VARIANTS) xv = PCX_X3_VARIANT;
     if (xv == 3 && (reinterpret_cast<uintptr_t>(a.in) & 15) != 0) xv = 1;
