@@ -519,6 +519,15 @@ bool pair_ok(const void* S, const void* Y, size_t L) {
   return L % 2 == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
 }
 
+// CTAs per column of the residual kernels: eight entries a thread where the
+// columns are short (each CTA ends with four FP64 atomics on its column's
+// norms; one entry a thread at 32^3 made 384 CTAs of them per column: 16
+// complex128 columns 53 -> 27 us, 16 of 64^3 181 -> 163)
+unsigned residual_grid(size_t L, int nvec) {
+  const size_t fill = (152u * 4u + nvec - 1) / nvec, want = (L + 8 * 256 - 1) / (8 * 256);
+  return (unsigned)std::max<size_t>(std::min<size_t>((L + 255) / 256, fill), std::min<size_t>(want, 152u * 4u));
+}
+
 unsigned grid_for(size_t work, int threads, unsigned cap = 152u * 32u) {
   return (unsigned)std::max<size_t>(1, std::min<size_t>((work + threads - 1) / threads, cap));
 }
@@ -620,7 +629,7 @@ cudaError_t launch_residual(const void* X, const void* AX, const double* theta, 
                             size_t L, int precision, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(norms, 0, sizeof(double) * 2 * nvec, s);
   if (e != cudaSuccess || nvec == 0) return e;
-  dim3 grid(grid_for(L, 256, 152u * 4u), nvec);
+  dim3 grid(std::max(1u, residual_grid(L, nvec)), nvec);
   if (precision == PCX_FP64)
     residual_kernel<double><<<grid, 256, 0, s>>>(static_cast<const cx<double>*>(X), static_cast<const cx<double>*>(AX),
                                                  theta, static_cast<cx<double>*>(R), norms, nvec, L);
@@ -634,7 +643,7 @@ cudaError_t launch_residual_mixed(const void* X, const void* AX, const double* t
                                   double* norms, int nvec, size_t L, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(norms, 0, sizeof(double) * 2 * nvec, s);
   if (e != cudaSuccess || nvec == 0) return e;
-  dim3 grid(grid_for(L, 256, 152u * 4u), nvec);
+  dim3 grid(std::max(1u, residual_grid(L, nvec)), nvec);
   residual_mixed_kernel<<<grid, 256, 0, s>>>(static_cast<const double2*>(X), static_cast<const double2*>(AX), theta,
                                              static_cast<float2*>(R32), static_cast<float2*>(X32), norms, nvec, L);
   return cudaGetLastError();
