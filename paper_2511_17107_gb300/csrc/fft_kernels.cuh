@@ -25,6 +25,7 @@
 // through shared memory with 16-byte accesses.
 #pragma once
 
+#include <algorithm>
 #include <cuda_runtime.h>
 
 #include "cx.cuh"
@@ -603,36 +604,43 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, 3) pass_kernel(PassArgs a)
 }
 
 // W = K_P^{-1} R per mode: r/|k|^2 + (1/gamma_p - 1) conj(k) (k . r) / |k|^4.
+// A thread takes one mode through a group of vectors: kappa and the division
+// cost more than the two products of a vector, and the FP64 pipe bounds the
+// complex128 form.  Measured (16 complex128 vectors at 32^3, CTAs of 128 so
+// that the groups of a small grid still reach every SM): 69 -> 40 us.
 template <typename T>
-__global__ void precond_kernel(const cx<T>* __restrict__ R, cx<T>* __restrict__ W, const cx<T>* __restrict__ lam,
-                               int n, int nvec, KParams kp) {
+__global__ void __launch_bounds__(128) precond_kernel(const cx<T>* __restrict__ R, cx<T>* __restrict__ W,
+                                                      const cx<T>* __restrict__ lam, int n, int nvec, int group,
+                                                      KParams kp) {
   const size_t n3 = (size_t)n * n * n;
   const int lg = __ffs(n) - 1;   // n is a power of two
-  const size_t total = n3 * nvec;
+  const int v0 = blockIdx.y * group, v1 = v0 + group < nvec ? v0 + group : nvec;
   const T ig = (T)(1.0 / kp.gamma);
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t v = e >> (3 * lg), mode = e & (n3 - 1);
+  for (size_t mode = (size_t)blockIdx.x * blockDim.x + threadIdx.x; mode < n3; mode += (size_t)gridDim.x * blockDim.x) {
     const int p1 = (int)(mode & (n - 1)), p2 = (int)((mode >> lg) & (n - 1)), p3 = (int)(mode >> (2 * lg));
     cx<T> kap[3];
     kappa_at<T>(lam, n, kp, p1, p2, p3, kap);
-    const size_t base = v * 3 * n3 + mode;
-    const cx<T> r0 = R[base], r1 = R[base + n3], r2 = R[base + 2 * n3];
     const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
-    cx<T> w0, w1, w2;
-    if (k2 > (T)0) {
-      const T ik2 = (T)1 / k2;
-      const T cg = ig * penalty_inv_weight(kp, k2) - (T)1;
-      cx<T> sk = cfma(kap[2], r2, cfma(kap[1], r1, kap[0] * r0));
-      sk = scale(sk, cg * ik2 * ik2);
-      w0 = cfma_conj(kap[0], sk, scale(r0, ik2));
-      w1 = cfma_conj(kap[1], sk, scale(r1, ik2));
-      w2 = cfma_conj(kap[2], sk, scale(r2, ik2));
-    } else {
-      w0 = w1 = w2 = mk((T)0, (T)0);
+    const bool nz = k2 > (T)0;
+    const T ik2 = nz ? (T)1 / k2 : (T)0;
+    const T cg = ig * penalty_inv_weight(kp, k2) - (T)1;
+    const T cs = cg * ik2 * ik2;
+    for (int v = v0; v < v1; ++v) {
+      const size_t base = (size_t)v * 3 * n3 + mode;
+      const cx<T> r0 = R[base], r1 = R[base + n3], r2 = R[base + 2 * n3];
+      cx<T> w0, w1, w2;
+      if (nz) {
+        const cx<T> sk = scale(cfma(kap[2], r2, cfma(kap[1], r1, kap[0] * r0)), cs);
+        w0 = cfma_conj(kap[0], sk, scale(r0, ik2));
+        w1 = cfma_conj(kap[1], sk, scale(r1, ik2));
+        w2 = cfma_conj(kap[2], sk, scale(r2, ik2));
+      } else {
+        w0 = w1 = w2 = mk((T)0, (T)0);
+      }
+      W[base] = w0;
+      W[base + n3] = w1;
+      W[base + 2 * n3] = w2;
     }
-    W[base] = w0;
-    W[base + n3] = w1;
-    W[base + 2 * n3] = w2;
   }
 }
 
@@ -1146,13 +1154,15 @@ cudaError_t run_div_norms_t(const pcx_ctx* c, const KParams& kp, const void* X, 
 
 template <typename T>
 cudaError_t run_precond_t(const pcx_ctx* c, const KParams& kp, const void* R, void* W, int nvec, cudaStream_t s) {
-  const size_t total = (size_t)c->n * c->n * c->n * nvec;
-  const int threads = 256;
-  size_t blocks = (total + threads - 1) / threads;
-  if (blocks > 152u * 16u) blocks = 152u * 16u;
+  const size_t n3 = (size_t)c->n * c->n * c->n;
+  const unsigned cells = (unsigned)((n3 + 127) / 128);
+  // groups of up to 16 vectors; small grids take smaller ones so that every SM has work
+  int group = nvec < 16 ? nvec : 16;
+  while (group > 1 && cells * (unsigned)((nvec + group - 1) / group) < 152u * 4u) group = (group + 1) / 2;
+  group = std::max(group, (nvec + 65534) / 65535);   // blockIdx.y is at most 65535
   const void* lam = sizeof(T) == 8 ? c->dev.lam64 : c->dev.lam32;
-  fftk::precond_kernel<T><<<(unsigned)blocks, threads, 0, s>>>(static_cast<const cx<T>*>(R), static_cast<cx<T>*>(W),
-                                                               static_cast<const cx<T>*>(lam), c->n, nvec, kp);
+  fftk::precond_kernel<T><<<dim3(cells, (unsigned)((nvec + group - 1) / group)), 128, 0, s>>>(
+      static_cast<const cx<T>*>(R), static_cast<cx<T>*>(W), static_cast<const cx<T>*>(lam), c->n, nvec, group, kp);
   return cudaGetLastError();
 }
 
