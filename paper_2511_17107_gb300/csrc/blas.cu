@@ -89,18 +89,6 @@ __global__ void __launch_bounds__(256) gram_kernel(const cx<T>* __restrict__ A, 
 }
 
 // ---------------------------------------------------------------------------
-// Double-float arithmetic on the FP32 pipes (GB300's FP64 rate is a small
-// fraction of its FP32 rate) for the complex128 combinations: every FP64
-// entry is split into FP32 hi + lo (about 48 significant bits); each real
-// product x*y is formed as hi*hi exactly (TwoProd with an FMA) plus the cross
-// terms, and accumulated in a double-float pair (Knuth's TwoSum), both
-// error-free transformations of Dekker (1971) and Knuth (TAOCP vol. 2).
-// __fadd_rn / __fmul_rn keep the compiler from fusing the steps.  Entries
-// must stay inside the FP32 exponent range. 
-// ---------------------------------------------------------------------------
-using dfloat::DF;
-
-// ---------------------------------------------------------------------------
 // Combine: Y_j = sum_i S_i C[i][j] (+ beta Y_j), one row per thread, up to
 // CY output columns per sweep; C staged in shared memory in T.
 // ---------------------------------------------------------------------------
@@ -248,61 +236,101 @@ __global__ void __launch_bounds__(256, 2) combine2_kernel(const float4* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Combine for complex128 on the FP32 pipes with FP64-level accuracy: the
-// split / TwoProd / TwoSum scheme above.  Each row's inputs
-// are split once and reused for the CY outputs of the sweep; C is split once
-// per CTA into shared memory.
+// Combine for complex128 on the FP32 pipes (GB300's FP64 rate is a small
+// fraction of its FP32 rate): entries and coefficients split into FP32 hi + lo
+// and sums kept as double-float pairs (dfloat.cuh).  Entries must stay inside
+// the FP32 exponent range.  Each row's entries are split once (integer
+// operations) for the CT outputs of the sweep; C is split once per CTA into
+// shared memory.  Packed operations take half the issue slots of scalar ones
+// and leave room for the splits; their pairs are the same part of two outputs,
+// so that a coefficient is read once for the real and the imaginary sums (with
+// (re, im) as the pair the reads of C took as long as the arithmetic).  Bound
+// by the FP32 pipes.
+// CT = 4, 8, 12 or 16 outputs, so that narrow sweeps (few active columns) don't
+// pay for 16.  Measured at 16 -> 16 columns of 3 128^3 rows: 3.09 ms with
+// scalar operations of the textbook form (13 a product; entries split by
+// truncation, whose error is a third larger), 2.54 now (FP32 pipes alone 1.9,
+// HBM 0.47); at 3 32^3 rows 72 -> 56 us, for 3 outputs 74 -> 25.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) combine_ff_kernel(const double2* __restrict__ S, int ns,
-                                                         const double* __restrict__ Cm, int ny, int j0, double beta,
-                                                         double2* __restrict__ Y, size_t L) {
+template <int CT>
+__global__ void __launch_bounds__(256) combine_ff_kernel(const double2* __restrict__ S, int ns,
+                                                                   const double* __restrict__ Cm, int ny, int j0,
+                                                                   int nyl, double beta, double2* __restrict__ Y,
+                                                                   size_t L) {
   extern __shared__ __align__(16) unsigned char csm[];
-  float4* c = reinterpret_cast<float4*>(csm);   // [ns][CY]: (re hi, re lo, im hi, im lo)
-  const int nyl = (ny - j0 < CY) ? ny - j0 : CY;
-  for (int e = threadIdx.x; e < ns * CY; e += blockDim.x) {
-    const int i = e / CY, j = e % CY;
-    float4 v = make_float4(0, 0, 0, 0);
-    if (j < nyl) {
-      const double re = Cm[2 * ((size_t)i * ny + j0 + j)], im = Cm[2 * ((size_t)i * ny + j0 + j) + 1];
-      dfloat::split(re, v.x, v.y);
-      dfloat::split(im, v.z, v.w);
-    }
-    c[e] = v;
+  float4* c = reinterpret_cast<float4*>(csm);   // [ns][CT / 2][2]: hi re, re', im, im'; lo the same
+  for (int e = threadIdx.x; e < ns * CT / 2; e += blockDim.x) {
+    const int i = e / (CT / 2), j = 2 * (e % (CT / 2));
+    float h[2][2] = {}, t[2][2] = {};   // [part][output]
+#pragma unroll
+    for (int o = 0; o < 2; ++o)
+      if (j + o < nyl)
+#pragma unroll
+        for (int p = 0; p < 2; ++p) dfloat::split_rn(Cm[2 * ((size_t)i * ny + j0 + j + o) + p], h[p][o], t[p][o]);
+    c[2 * e] = make_float4(h[0][0], h[0][1], h[1][0], h[1][1]);
+    c[2 * e + 1] = make_float4(t[0][0], t[0][1], t[1][0], t[1][1]);
   }
   __syncthreads();
   for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < L; l += (size_t)gridDim.x * blockDim.x) {
-    DF re[CY], im[CY];
+    float2 re[CT / 2], im[CT / 2], rr[CT / 2], ir[CT / 2];   // sums of two outputs and their compensations
 #pragma unroll
-    for (int j = 0; j < CY; ++j) re[j] = im[j] = DF{0.f, 0.f};
+    for (int j = 0; j < CT / 2; ++j) re[j] = im[j] = rr[j] = ir[j] = make_float2(0.f, 0.f);
+    double2 next = S[l];
+#pragma unroll 1
     for (int i = 0; i < ns; ++i) {
-      const double2 sv = S[(size_t)i * L + l];
-      float sr, srl, si, sil;   // integer splits: no FP64 instruction in the loop
-      dfloat::split(sv.x, sr, srl);
-      dfloat::split(sv.y, si, sil);
+      const double2 sv = next;
+      if (i + 1 < ns) next = S[(size_t)(i + 1) * L + l];
+      float h, t;
+      dfloat::split_rn(sv.x, h, t);
+      const float2 xh = make_float2(h, h), xl = make_float2(t, t);
+      dfloat::split_rn(sv.y, h, t);
+      const float2 yh = make_float2(h, h), yl = make_float2(t, t), nh = make_float2(-h, -h), nl = make_float2(-t, -t);
 #pragma unroll
-      for (int j = 0; j < CY; ++j) {
-        const float4 cv = c[i * CY + j];
-        // s c: re = sr cr - si ci, im = sr ci + si cr
-        dfloat::mac2<false>(re[j], sr, srl, cv.x, cv.y);
-        dfloat::mac2<true>(re[j], si, sil, cv.z, cv.w);
-        dfloat::mac2<false>(im[j], sr, srl, cv.z, cv.w);
-        dfloat::mac2<false>(im[j], si, sil, cv.x, cv.y);
+      for (int j = 0; j < CT / 2; ++j) {
+        const float4 ch = c[(i * (CT / 2) + j) * 2], cl = c[(i * (CT / 2) + j) * 2 + 1];
+        const float2 rh = make_float2(ch.x, ch.y), ih = make_float2(ch.z, ch.w);
+        const float2 rl = make_float2(cl.x, cl.y), il = make_float2(cl.z, cl.w);
+        dfloat::mac_pair(re[j], rr[j], xh, xl, rh, rl);
+        dfloat::mac_pair(re[j], rr[j], nh, nl, ih, il);
+        dfloat::mac_pair(im[j], ir[j], xh, xl, ih, il);
+        dfloat::mac_pair(im[j], ir[j], yh, yl, rh, rl);
       }
     }
 #pragma unroll
-    for (int j = 0; j < CY; ++j) {
+    for (int j = 0; j < CT; ++j) {
       if (j < nyl) {
         double2* yp = Y + (size_t)(j0 + j) * L + l;
-        double2 r = make_double2((double)re[j].s + (double)re[j].c, (double)im[j].s + (double)im[j].c);
+        const float2 a = re[j / 2], b = im[j / 2], ar = rr[j / 2], br = ir[j / 2];
+        double2 v = j % 2 ? make_double2((double)a.y + (double)ar.y, (double)b.y + (double)br.y)
+                          : make_double2((double)a.x + (double)ar.x, (double)b.x + (double)br.x);
         if (beta != 0.0) {
           const double2 y0 = *yp;
-          r.x += beta * y0.x;
-          r.y += beta * y0.y;
+          v.x += beta * y0.x;
+          v.y += beta * y0.y;
         }
-        *yp = r;
+        *yp = v;
       }
     }
   }
+}
+
+template <int CT>
+cudaError_t run_combine_ff(const void* S, int ns, const double* C, int ny, int j0, int nyl, double beta, void* Y,
+                           size_t L, cudaStream_t s) {
+  const size_t smem = (size_t)ns * CT * sizeof(float4);
+  if (smem > 48 * 1024) {
+    cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(combine_ff_kernel<CT>), smem);
+    if (e != cudaSuccess) return e;
+  }
+  // CTAs of 64 threads even out the short columns (32^3 has 20 warps of rows
+  // per SM); with many columns S_i the coefficients of a CTA leave room for few
+  // CTAs, so these are larger.  24 CTAs of 64 per SM divide evenly over any
+  // usual number of resident ones.
+  const unsigned threads = smem > 32 * 1024 ? 256 : 64;
+  const unsigned blocks = (unsigned)std::min<size_t>((L + threads - 1) / threads, 152u * 24u * 64u / threads);
+  combine_ff_kernel<CT><<<blocks, threads, smem, s>>>(static_cast<const double2*>(S), ns, C, ny, j0, nyl, beta,
+                                                         static_cast<double2*>(Y), L);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -575,18 +603,22 @@ cudaError_t launch_gram_cuda_cores(const void* A, int na, const void* B, int nb,
 cudaError_t launch_combine(const void* S, int ns, const double* C, int ny, double beta, void* Y, size_t L,
                            int precision, cudaStream_t s) {
   if (L == 0) return cudaSuccess;
+  if (precision == PCX_FP64) {
+    // sweeps of equal width, at most 16 outputs each
+    const int sweeps = (ny + 15) / 16, width = sweeps ? (ny + sweeps - 1) / sweeps : 0;
+    for (int j0 = 0; j0 < ny; j0 += width) {
+      const int nyl = std::min(width, ny - j0);
+      auto run = nyl <= 4 ? run_combine_ff<4> : nyl <= 8 ? run_combine_ff<8> : nyl <= 12 ? run_combine_ff<12>
+                                                                                        : run_combine_ff<16>;
+      cudaError_t e = run(S, ns, C, ny, j0, nyl, beta, Y, L, s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   const int threads = 256;
   const unsigned blocks = grid_for(L, threads, 152u * 8u);
   for (int j0 = 0; j0 < ny; j0 += CY) {
-    if (precision == PCX_FP64) {
-      const size_t smem = (size_t)ns * CY * sizeof(float4);
-      if (smem > 48 * 1024) {
-        cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(combine_ff_kernel), smem);
-        if (e != cudaSuccess) return e;
-      }
-      combine_ff_kernel<<<grid_for(L, 128, 152u * 16u), 128, smem, s>>>(static_cast<const double2*>(S), ns, C, ny,
-                                                                         j0, beta, static_cast<double2*>(Y), L);
-    } else if (pair_ok(S, Y, L)) {
+    if (pair_ok(S, Y, L)) {
       const size_t smem = (size_t)(RING * 256 + ns * CY) * sizeof(float4);
       cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(combine2_kernel<false>), smem);
       if (e != cudaSuccess) return e;
