@@ -6,11 +6,11 @@
 //
 // Every column gets an exponent E (|re|, |im| < 2^E over the rows seen so
 // far) and its entries become signed fixed-point integers of 49 bits below
-// 2^E, cut into NS = 5 balanced digits of base 2^10.  A digit lies in
+// 2^E, cut into five balanced digits of base 2^10.  A digit lies in
 // [-512, 512] and is exact in half precision, so the product of two digit
 // columns on mma.sync (FP16 operands, FP32 accumulators) is a sum of integers
 // of at most 2^18.  Digit pairs (i, j) of one weight g = i + j share an
-// accumulator; pairs beyond NS - 1 are left out.  Over the KC = 32 rows of a
+// accumulator; pairs beyond g = 4 are left out.  Over the KC = 32 rows of a
 // chunk the sums of groups 0 and 1 are at most 2^24 and exact; those of later
 // groups could pass 2^24 only where all digits are near their limit in every
 // row, and round by units 2^-38 and less then.  The chunk sums are added into
@@ -56,7 +56,13 @@ namespace {
 
 constexpr int KC = 32;                 // rows per chunk
 constexpr int MAXC = 48;               // columns of A or B per launch
+constexpr int NS = 5;                  // digits
 constexpr int DB = 10;                 // bits per digit
+constexpr int MB = DB - 1 + DB * (NS - 1);   // magnitude bits of the fixed-point value
+// digit group 0 has weight 2^SUM_BITS in the 64-bit sums: the last group sits
+// 10 bits below the unit and is rounded into it, so that MAX_ROWS rows cannot
+// overflow
+constexpr int SUM_BITS = DB * (NS - 2);
 constexpr long long MAX_ROWS = 16000;  // rows per CTA: 500 chunks of at most 2^53 keep the 64-bit sums in range
 constexpr int E_MIN = 128;             // smallest exponent of a complex128 column (biased): keeps 2^(MB - E) finite
 
@@ -75,15 +81,6 @@ struct Entry<float> {
   static constexpr int BAD = 255;
 };
 
-template <int NS>
-struct Digits {
-  static constexpr int MB = DB - 1 + DB * (NS - 1);   // magnitude bits of the fixed-point value
-  // weight of digit group 0 in the 64-bit sums is 2^S; with NS = 5 the last
-  // group sits 10 bits below the unit and is rounded into it, so that MAX_ROWS
-  // rows cannot overflow
-  static constexpr int S = NS == 5 ? 30 : DB * (NS - 1);
-};
-
 __device__ __forceinline__ int exp_bits(double a, double b) {
   const uint32_t x = (uint32_t)(__double_as_longlong(a) >> 32) & 0x7fffffffu;
   const uint32_t y = (uint32_t)(__double_as_longlong(b) >> 32) & 0x7fffffffu;
@@ -98,13 +95,12 @@ __device__ __forceinline__ int exp_bits(float a, float b) {
 //
 // complex128: one FMA against 1.5 2^52 rounds v 2^(MB - E) to an integer in
 // the low mantissa bits; half a base added to every digit balances them.
-template <int NS>
 struct Fields64 {
   template <int I>
   static __device__ __forceinline__ constexpr bool leading() { return I == 0; }
   uint32_t lo, hi;
   __device__ __forceinline__ Fields64(double v, double scale) {
-    // 1.5 2^52 + sum_i 512 1024^i over all NS digits
+    // 1.5 2^52 + sum_i 512 1024^i over all digits
     constexpr double magic =
         6755399441055744.0 + (double)((1ll << (DB - 1)) * (((1ll << (DB * NS)) - 1) / ((1 << DB) - 1)));
     const unsigned long long u = (unsigned long long)__double_as_longlong(fma(v, scale, magic));
@@ -123,53 +119,38 @@ struct Fields64 {
 };
 // complex64: the leading two digits by an FMA against 1.5 2^23, then two
 // digits at a time of the exact remainder
-template <int NS>
 struct Fields32 {
   template <int I>
   static __device__ __forceinline__ constexpr bool leading() { return (I & 1) == 0; }
-  uint32_t w[3];
+  uint32_t w[3];   // two digits each (the leading one at bit DB), the last word one
   static constexpr uint32_t HALF2 = (1u << (DB - 1)) * ((1u << DB) + 1);   // half a base in two digits
   __device__ __forceinline__ Fields32(float v, float2 scale) {
     constexpr float magic = 12582912.f;
     float r = v * scale.x * scale.y;   // |r| < 2^MB
-    constexpr float unit0 = (float)(1ll << (DB * (NS - 2)));   // unit of the leading word
+    constexpr float unit0 = (float)(1ll << (DB * (NS - 2))), unit1 = (float)(1 << DB);   // units of the words
     const float t0 = fmaf(r, 1.f / unit0, magic);
     r = fmaf(t0 - magic, -unit0, r);
     w[0] = __float_as_uint(t0) + HALF2;
-    if constexpr (NS == 3) {
-      w[1] = __float_as_uint(r + (magic + (float)(1 << (DB - 1))));
-    } else if constexpr (NS == 4) {
-      w[1] = __float_as_uint(r + magic) + HALF2;
-    } else {
-      constexpr float unit1 = (float)(1 << DB);
-      const float t1 = fmaf(r, 1.f / unit1, magic);
-      r = fmaf(t1 - magic, -unit1, r);
-      w[1] = __float_as_uint(t1) + HALF2;
-      w[2] = __float_as_uint(r + (magic + (float)(1 << (DB - 1))));
-    }
+    const float t1 = fmaf(r, 1.f / unit1, magic);
+    r = fmaf(t1 - magic, -unit1, r);
+    w[1] = __float_as_uint(t1) + HALF2;
+    w[2] = __float_as_uint(r + (magic + (float)(1 << (DB - 1))));
   }
   template <int I>
   __device__ __forceinline__ uint32_t field() const {
-    // words hold two digits each (the leading one at bit DB), the last of an odd NS one
-    if constexpr (I == NS - 1 && (NS & 1)) return w[NS / 2];
+    if constexpr (I == NS - 1) return w[NS / 2];
     else return (I & 1) ? w[I / 2] : w[I / 2] >> DB;
   }
 };
-template <typename T, int NS>
-struct FieldsOf;
-template <int NS>
-struct FieldsOf<double, NS> { using type = Fields64<NS>; };
-template <int NS>
-struct FieldsOf<float, NS> { using type = Fields32<NS>; };
+template <typename T>
+using Fields = std::conditional_t<sizeof(T) == 8, Fields64, Fields32>;
 // 2^(MB - (E - BIAS)); as two factors for complex64, where one could not
 // reach far enough
-template <int NS>
 __device__ __forceinline__ double scale_of(double, int E) {
-  return __hiloint2double((1023 + Digits<NS>::MB + Entry<double>::BIAS - E) << 20, 0);
+  return __hiloint2double((1023 + MB + Entry<double>::BIAS - E) << 20, 0);
 }
-template <int NS>
 __device__ __forceinline__ float2 scale_of(float, int E) {
-  const int sh = Digits<NS>::MB + Entry<float>::BIAS - E, s1 = sh < 100 ? sh : 100;
+  const int sh = MB + Entry<float>::BIAS - E, s1 = sh < 100 ? sh : 100;
   return make_float2(__int_as_float((127 + s1) << 23), __int_as_float((127 + sh - s1) << 23));
 }
 
@@ -231,7 +212,7 @@ struct DigitArgs {
 // per SM.  REG > 0: the multiplying warps take REG registers and the cutting
 // warps give them up (MW = SW = 8 at 128 each: REG + cut_regs = 256).
 
-template <typename TA, typename TB, int NS, int MW, int SW, int MT, int CTAS, int REG>
+template <typename TA, typename TB, int MW, int SW, int MT, int CTAS, int REG>
 __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(DigitArgs g) {
   static_assert(REG == 0 || (MW == 8 && SW == 8 && CTAS == 1 && REG % 8 == 0), "register split");
   using CA = typename Entry<TA>::C;
@@ -291,7 +272,7 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
     auto cut_cols = [&](auto* entries, int ncol, int npair, int f, int x0, int row0, int n8, unsigned char* buf) {
       using C = std::remove_const_t<std::remove_pointer_t<decltype(entries)>>;
       using T = decltype(C::x);
-      using F = typename FieldsOf<T, NS>::type;
+      using F = Fields<T>;
       constexpr int NB = 2;
       const int* eold = expo + ((f + 2) % 3) * 2 * MAXC + x0;
       int* enew = expo + (f % 3) * 2 * MAXC + x0;
@@ -322,7 +303,7 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
             if (E[b] != old[b]) changed[f % 3] = 1;
             if (isbad) bad[x0 + c] = 1;
           }
-          const auto sc = scale_of<NS>((T)0, E[b]);
+          const auto sc = scale_of((T)0, E[b]);
 #pragma unroll
           for (int part = 0; part < 2; ++part) {
             const F f0(part ? v[b][0].y : v[b][0].x, sc), f1(part ? v[b][1].y : v[b][1].x, sc);
@@ -447,13 +428,11 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
       for (int i = 0; i < 8; ++i) {
         long long t = v[k][i];
 #pragma unroll
-        for (int w = 0; w < NS; ++w) {
-          if (NS == 5 && w == NS - 1) continue;
+        for (int w = 0; w < NS - 1; ++w) {
           // the unit of the 64-bit sums is that of group 3: the last of five
           // groups joins it as a fraction and is rounded with it
-          const float xf = NS == 5 && w == 3 ? fmaf(acc[NS - 1][i], 1.f / (float)(1 << DB), acc[w][i]) : acc[w][i];
-          const int sh = Digits<NS>::S - DB * w;
-          t += (long long)__float2int_rn(xf) * (1ll << (sh >= 0 ? sh : 0));
+          const float xf = w == NS - 2 ? fmaf(acc[NS - 1][i], 1.f / (float)(1 << DB), acc[w][i]) : acc[w][i];
+          t += (long long)__float2int_rn(xf) * (1ll << (SUM_BITS - DB * w));
         }
         v[k][i] = t;
       }
@@ -471,7 +450,7 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
       const int r = tr * 16 + gid + 8 * ((i >> 1) & 1), c = tc * 16 + 8 * (i >> 2) + 2 * tg + (i & 1);
       const int sa = slot_a(r), sb = slot_b(c);
       double d = ldexp((double)v[k][i], expo[ef + sa] - Entry<TA>::BIAS + expo[ef + sb] - Entry<TB>::BIAS -
-                                            (Digits<NS>::S + 2 * (DB - 1)));
+                                            (SUM_BITS + 2 * (DB - 1)));
       if (bad[sa] | bad[sb]) d = __longlong_as_double(0x7ff8000000000000LL);
       out[(size_t)r * rb + c] = d;
     }
@@ -528,9 +507,9 @@ StreamScratch& dscratch() {
   return s;
 }
 
-template <typename TA, typename TB, int NS, int MW, int SW, int MT, int CTAS, int REG>
+template <typename TA, typename TB, int MW, int SW, int MT, int CTAS, int REG>
 cudaError_t run_block(DigitArgs g, int sms, double* G, int ldg, cudaStream_t s) {
-  auto kern = gram_digits_kernel<TA, TB, NS, MW, SW, MT, CTAS, REG>;
+  auto kern = gram_digits_kernel<TA, TB, MW, SW, MT, CTAS, REG>;
   const int rtot = 2 * g.na8 + (g.sym ? 0 : 2 * g.nb8);
   const size_t smem = (size_t)2 * NS * rtot * 64 + (size_t)2 * ((g.na + 1) / 2) * 64 * sizeof(typename Entry<TA>::C) +
                       (g.sym ? 0 : (size_t)2 * ((g.nb + 1) / 2) * 64 * sizeof(typename Entry<TB>::C)) +
@@ -566,7 +545,7 @@ cudaError_t run_block(DigitArgs g, int sms, double* G, int ldg, cudaStream_t s) 
   return cudaGetLastError();
 }
 
-template <typename TA, typename TB, int NS>
+template <typename TA, typename TB>
 cudaError_t run_digits(const void* A, int na, const void* B, int nb, size_t L, double* G, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -590,11 +569,11 @@ cudaError_t run_digits(const void* A, int na, const void* B, int nb, size_t L, d
       const int tr = 2 * g.na8 / 16, tc = 2 * g.nb8 / 16;
       const int items = g.sym ? tr * (tr + 1) / 2 : tr * tc;
       // tiles per multiplying warp
-      if (items <= 4) e = run_block<TA, TB, NS, 4, 4, 1, 2, 0>(g, sms, out, nb, s);
-      else if (items <= 8) e = run_block<TA, TB, NS, 4, 4, 2, 2, 0>(g, sms, out, nb, s);
-      else if (items <= 16) e = run_block<TA, TB, NS, 8, 8, 2, 1, 144>(g, sms, out, nb, s);
-      else if (items <= 24) e = run_block<TA, TB, NS, 8, 8, 3, 1, 152>(g, sms, out, nb, s);
-      else e = run_block<TA, TB, NS, 8, 8, 5, 1, 184>(g, sms, out, nb, s);
+      if (items <= 4) e = run_block<TA, TB, 4, 4, 1, 2, 0>(g, sms, out, nb, s);
+      else if (items <= 8) e = run_block<TA, TB, 4, 4, 2, 2, 0>(g, sms, out, nb, s);
+      else if (items <= 16) e = run_block<TA, TB, 8, 8, 2, 1, 144>(g, sms, out, nb, s);
+      else if (items <= 24) e = run_block<TA, TB, 8, 8, 3, 1, 152>(g, sms, out, nb, s);
+      else e = run_block<TA, TB, 8, 8, 5, 1, 184>(g, sms, out, nb, s);
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
@@ -606,8 +585,8 @@ cudaError_t launch_gram_digits(const void* A, int na, const void* B, int prec_b,
                                cudaStream_t s) {
   if (na < 1 || nb < 1 || !A || !B) return cudaErrorInvalidValue;
   if (L == 0) return cudaMemsetAsync(G, 0, sizeof(double) * 2 * (size_t)na * nb, s);
-  return prec_b == PCX_FP64 ? run_digits<double, double, 5>(A, na, B, nb, L, G, s)
-                            : run_digits<double, float, 5>(A, na, B, nb, L, G, s);
+  return prec_b == PCX_FP64 ? run_digits<double, double>(A, na, B, nb, L, G, s)
+                            : run_digits<double, float>(A, na, B, nb, L, G, s);
 }
 
 void gram_digits_release_stream(cudaStream_t s) { dscratch().release(s); }
