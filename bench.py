@@ -48,10 +48,10 @@ METRIC = "compensated-operator applies/s at 128^3"
 # DRAM bytes of one vector through the pass kernels at 16 vectors per
 # launch: dram__bytes_read.sum + dram__bytes_write.sum of the launches of one
 # chunk in an ncu capture of this benchmark, divided by 16; keyed by the pass
-# structure and, for the three-pass chain, pass B's kernel variant (one tile
-# per CTA, or the warp-specialised one); the x-pass variants move the same
+# structure and, for the three-pass chain, pass B's kernel variant (at N = 128
+# both settings run one tile per CTA); the x-pass variants move the same
 # bytes.  Used only when the run uses that chunk, structure and variant.
-TRAFFIC_BYTES_PER_VECTOR_128_C64 = {(5, None): 8.8128e9 / 16, (3, 0): 5.321861e9 / 16, (3, 1): 5.304722e9 / 16}
+TRAFFIC_BYTES_PER_VECTOR_128_C64 = {(5, None): 8.8128e9 / 16, (3, 0): 5.286857e9 / 16, (3, 1): 5.286857e9 / 16}
 TRAFFIC_CHUNK = 16
 UNIT = "vector-applies/s"
 

@@ -1,6 +1,6 @@
 // Autotuner of the apply launch configuration: the pass structure (five
 // passes, or the three-pass form where it exists), vectors per launch chunk
-// (how much of the block sweeps the passes while L2-resident), the kernel
+// (how much of the block goes through a pass in one launch), the kernel
 // variants of the three-pass chain's x and z passes, and whether the launch
 // chain replays as a CUDA graph.  Each candidate is timed
 // with CUDA events on the caller's stream; the choice is cached per
