@@ -607,7 +607,9 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, 3) pass_kernel(PassArgs a)
 // A thread takes one mode through a group of vectors: kappa and the division
 // cost more than the two products of a vector, and the FP64 pipe bounds the
 // complex128 form.  Measured (16 complex128 vectors at 32^3, CTAs of 128 so
-// that the groups of a small grid still reach every SM): 69 -> 40 us.
+// that the groups of a small grid still reach every SM): 69 -> 40 us. At 128^3,
+// 16 vectors: complex64 406 -> 266 us, complex128 4.32 -> 2.00 ms; one vector 46
+// -> 38 and 279 -> 285 us.
 template <typename T>
 __global__ void __launch_bounds__(128) precond_kernel(const cx<T>* __restrict__ R, cx<T>* __restrict__ W,
                                                       const cx<T>* __restrict__ lam, int n, int nvec, int group,
@@ -1155,7 +1157,9 @@ cudaError_t run_div_norms_t(const pcx_ctx* c, const KParams& kp, const void* X, 
 template <typename T>
 cudaError_t run_precond_t(const pcx_ctx* c, const KParams& kp, const void* R, void* W, int nvec, cudaStream_t s) {
   const size_t n3 = (size_t)c->n * c->n * c->n;
-  const unsigned cells = (unsigned)((n3 + 127) / 128);
+  // at most 32 CTAs per SM, whose threads go on to further modes: one mode per
+  // thread made a single vector of 128^3 76 us instead of 38 (complex64)
+  const unsigned cells = (unsigned)std::min<size_t>((n3 + 127) / 128, 152u * 32u);
   // groups of up to 16 vectors; small grids take smaller ones so that every SM has work
   int group = nvec < 16 ? nvec : 16;
   while (group > 1 && cells * (unsigned)((nvec + group - 1) / group) < 152u * 4u) group = (group + 1) / 2;
