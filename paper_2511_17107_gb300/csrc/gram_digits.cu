@@ -338,6 +338,7 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
       const unsigned char* rf = raw + (f & 1) * raw_bytes;
       cut_cols(reinterpret_cast<const CA*>(rf), g.na, pa, f, 0, 0, g.na8, buf);
       cut_cols(reinterpret_cast<const CB*>(rf + rawa_bytes), g.nb, pb, f, MAXC, ra, g.nb8, buf);
+      __syncwarp();   // the exponents just written by two lanes are read by the whole warp in the next chunk
       bar_arrive<THREADS>(BAR_FULL + (f & 1));
       fetch(f + 2);   // into the slots just read
     }

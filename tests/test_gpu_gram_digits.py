@@ -95,6 +95,19 @@ def test_ranges(pcx, kind, mixed):
         _check(a, a, _gram(pcx, a, a))
 
 
+@pytest.mark.parametrize("row", [31, 32, 63, 64, 96])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_exponent_steps_between_chunks(pcx, row, mixed):
+    """A column's scale jumps 2^40-fold at one row (chunks hold 32) and stays: every lane that cuts the column has
+    to see the new exponent in the next chunk, from the first to the second one too."""
+    for na, nb in ((1, 1), (16, 16), (48, 31)):
+        a = _block("plain", na, 128, np.complex128, 8)
+        b = _block("plain", nb, 128, np.complex64 if mixed else np.complex128, 9)
+        a[:, row:] *= 2.0 ** 40
+        b[:, row:] *= 2.0 ** 40
+        _check(a, b, _gram(pcx, a, b))
+
+
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
 def test_non_finite(pcx, value):
     a = _block("plain", 9, 300, np.complex128, 6)
