@@ -271,6 +271,22 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
   double lrn_best = INFINITY;
   int no_drop = 0;
   res.assign(n, INFINITY);
+  // The eigenvalues of an FP64 run are the Rayleigh quotients x^H AX / x^H x
+  // of the block it returns, off by |residual|^2 / gap.  The Ritz values that
+  // the last step took from an ill-conditioned [X P W] carry the rounding of
+  // its Gram matrices divided by their smallest eigenvalue: up to 1e-9
+  // relative with 10th-order stencils, and the image AX that the steps carry
+  // along adds its own.  One apply and one n x n product per solve.
+  auto quotients = [&](const std::vector<double>& nrm) -> pcx_status {
+    if (run.prec != PCX_FP64) return PCX_OK;
+    CK(run.apply(run.S.p, run.AS.p, n));
+    std::vector<cd> g;
+    pcx_status s2 = run.gram(run.S.p, n, run.AS.p, n, g);
+    if (s2 != PCX_OK) return s2;
+    for (int j = 0; j < n; ++j) theta[j] = g[(size_t)j * n + j].real() / nrm[n + j];
+    std::sort(theta.begin(), theta.end());
+    return PCX_OK;
+  };
   for (iters = 0;; ++iters) {
     // residual R = AX - X theta and norms
     CK(cudaMemcpyAsync(run.theta.p, theta.data(), sizeof(double) * n, cudaMemcpyHostToDevice, run.s));
@@ -293,7 +309,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
       std::fprintf(stderr, "[pcx] %s it %d worst %.3e theta0 %.12g theta_top %.4e\n",
                    run.prec == PCX_FP64 ? "fp64" : "fp32", iters, worst, theta[0], run.theta_top);
     }
-    if (worst <= tol) return PCX_OK;
+    if (worst <= tol) return quotients(nrm);
     if (worst <= stop_tol) {
       stopped_early = true;
       return PCX_OK;
@@ -313,7 +329,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
       stopped_early = true;
       return PCX_OK;
     }
-    if (iters >= maxit) return PCX_ENOCONV;
+    if (iters >= maxit) return (st = quotients(nrm)) != PCX_OK ? st : PCX_ENOCONV;
     Learned* lrn = run.learned;
     // learned correction: back to the base preconditioner once the worst
     // residual has not dropped 10% below its best for `patience` iterations
