@@ -466,11 +466,14 @@ pcx_status pcx_precond(pcx_ctx* ctx, const double k[3], double gamma, const void
  * the tensor cores (tcgen05 TF32 with hi/lo error compensation) or the
  * FP32 pipes (register-blocked FMAs, double-float sums across chunks), for
  * na, nb <= 64, even L and 16-byte aligned A, B; a generic CUDA-core
- * kernel otherwise.  PCX_FP64: 49-bit fixed-point entries below each
- * column's largest, multiplied exactly as integer digits on the tensor cores
- * (about 1e-15 of ||A_i|| ||B_j||), per-block partials summed in FP64; a
- * column with Inf or NaN gives NaN in its row or column of G.
- * 1 <= na, nb <= 128.
+ * kernel otherwise.  PCX_FP64: integer digits on the tensor cores.  In every
+ * 32 rows the entries of a column are taken as fixed-point numbers of 49 bits
+ * below their largest part, M_c; digit products are exact, those below the
+ * 50th bit left out, the sums kept in double-float and per-block partials
+ * summed in FP64.  Error of G_ij: about 2^-47.5 sqrt(sum_l (M_c M'_c)^2) plus
+ * 2^-47 sum_l |a_l||b_l| at most -- 2e-17 to 2e-14 of ||A_i|| ||B_j|| for
+ * columns even or falling off with the mode.  A column with Inf or NaN gives
+ * NaN in its row or column of G.  1 <= na, nb <= 128.
  */
 pcx_status pcx_gram(pcx_ctx* ctx, const void* A, int na, const void* B, int nb, size_t L,
                     int precision, void* G, void* stream);
@@ -495,8 +498,8 @@ int pcx_get_gram_path(void);
  * DEVICE buffer G (G[i*nb + j], interleaved doubles).  The X rows of the
  * Rayleigh-Ritz matrices in the mixed-precision refinement (Sec. 4: LOBPCG
  * with the block X held in FP64 and the search directions in FP32).
- * Accuracy: about 5e-15 of ||A_i|| ||B_j|| (integer digits on the tensor
- * cores, as pcx_gram with PCX_FP64).  A column with Inf or NaN gives NaN in
+ * Accuracy: that of pcx_gram with PCX_FP64 (integer digits on the tensor
+ * cores).  A column with Inf or NaN gives NaN in
  * its row or column of G.  A, B, G
  * 16-byte aligned device pointers; 1 <= na, nb <= 128.  Uses a per-device
  * scratch buffer owned by the library: concurrent calls on different streams

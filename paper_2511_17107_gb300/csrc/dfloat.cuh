@@ -98,5 +98,13 @@ __device__ __forceinline__ void add(DF& acc, float p, float e) {
   acc.c = __fadd_rn(acc.c, __fadd_rn(err, e));
 }
 
+// (s, c) <- (s + c, the rounding error of that sum): the compensation stays at
+// half an ulp of s (Fast2Sum; |c| <= |s| or s = 0 here).
+__device__ __forceinline__ void renorm(DF& a) {
+  const float s = __fadd_rn(a.s, a.c);
+  a.c = __fsub_rn(a.c, __fsub_rn(s, a.s));
+  a.s = s;
+}
+
 }  // namespace dfloat
 }  // namespace pcx

@@ -1,25 +1,36 @@
 // Gram products G = A^H B (Sec. 4: the Rayleigh-Ritz matrices of LOBPCG) with
 // A complex128 and B complex128 or complex64, by integer digits on the tensor
-// cores, accurate to the digits kept below each column's largest entry.
-// The mixed product gives the rows X^H [P W] of the refinement, whose entries
-// are far below the FP32 rounding of the products.
+// cores (splitting a product into exact tensor-core products: Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59 (2012) 95; Mukunoki et al., ISC High
+// Performance 2020).  The mixed product gives the rows X^H [P W] of the
+// refinement, whose entries are far below the FP32 rounding of the products.
 //
-// Every column gets an exponent E (|re|, |im| < 2^E over the rows seen so
-// far) and its entries become signed fixed-point integers of 49 bits below
-// 2^E, cut into five balanced digits of base 2^10.  A digit lies in
-// [-512, 512] and is exact in half precision, so the product of two digit
+// In every chunk of KC = 32 rows a column gets an exponent E (|re|, |im| <
+// 2^E in the chunk) and its entries become signed fixed-point integers of 49
+// bits below 2^E, cut into five balanced digits of base 2^10.  A digit lies
+// in [-512, 512] and is exact in half precision, so the product of two digit
 // columns on mma.sync (FP16 operands, FP32 accumulators) is a sum of integers
 // of at most 2^18.  Digit pairs (i, j) of one weight g = i + j share an
-// accumulator; pairs beyond g = 4 are left out.  Over the KC = 32 rows of a
-// chunk the sums of groups 0 and 1 are at most 2^24 and exact; those of later
-// groups could pass 2^24 only where all digits are near their limit in every
-// row, and round by units 2^-38 and less then.  The chunk sums are added into
-// 64-bit integers of unit 2^-48.  What is lost is the rounding of the entries
-// (2^-50 of the column's largest), the pairs left out and the last group's
-// fraction: 1e-15 of ||A_i|| ||B_j|| measured, 5e-15 with complex64 B,
-// against 5e-15 to 2e-13 for sums in double-float (splitting a product into
-// exact tensor-core products: Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
-// 59 (2012) 95; Mukunoki et al., ISC High Performance 2020).
+// accumulator; pairs beyond g = 4 are left out.  Over the rows of a chunk the
+// sums of groups 0 and 1 are at most 2^24 and exact; those of later groups
+// could pass 2^24 only where all digits are near their limit in every row,
+// and round by units 2^-38 and less then.  The chunk sums join double-float
+// sums (FP32 pairs) whose unit follows the columns' largest exponents so far.
+//
+// Accuracy.  The pairs left out and the rounding of the entries come to 2^-50
+// 2^(Ea + Eb) rms in a product of two reals, so an entry of G is off by about
+// 2^-47.5 sqrt(sum over rows of (M_c M'_c)^2), M_c the largest part of the
+// column in the row's chunk, and each chunk's addition rounds 2^-49 of the
+// running sum.  Exponents per chunk, and sums that float, keep columns that
+// are graded against each other accurate (A falling and B rising, so that all
+// rows weigh alike): only what falls inside 32 rows counts.  Largest error of
+// G over ||A_i|| ||B_j||, 16 x 43 columns of 3 128^3 rows falling off with
+// the mode as |p|^-power (powers of A, B), double-float sums / this kernel:
+// (0, 0) 4.8e-16 / 2e-17, (1, 1) 2.6e-15 / 1.2e-16, (2, 2) 1.3e-13 / 5.8e-15,
+// (4, 4) 1.1e-13 / 1.6e-14, (2, 0) 4.3e-16 / 2.8e-17; complex64 B (2, 2)
+// 2.2e-12 / 4.9e-15.  Over sum |a||b| with opposite powers (2, -2) 6.1e-16 /
+// 5e-17, (4, -4) 6.4e-16 / 2.4e-14, and one entry 1000 times all others in
+// both columns 5e-15 / 8e-15 (1.4e-14 at 3 64^3).
 //
 // The complex product is a real one over stacked columns, D = [Ar Ai]^T
 // [Br Bi]: Re G = D[i][j] + D[n+i][m+j], Im G = D[i][m+j] - D[n+i][j].  For
@@ -35,11 +46,13 @@
 //
 // What bounds it at 48 x 48: the multiplying warps (mma.sync peaks at 1,036
 // multiply-adds per clock and SM, measured; the kernel reaches half of it,
-// the rest is the conversion of the chunk sums to integers at 16 a clock and
-// SM); narrow products are bound by the cutting warps.  Measured at 3 128^3
-// rows (GB300): complex128 48 x 48 30.5 ms in double-float on the FP32 pipes,
-// 6.6 ms here; 16 x 16 3.46 and 1.5 ms; complex128 x complex64 16 x 32 4.94
-// and 2.1 ms.
+// the rest is the addition of the chunk sums, 20 FP32 operations each); narrow
+// products are bound by the cutting warps.  Measured at 3 128^3 rows (GB300):
+// complex128 48 x 48 30.4 ms in double-float on the FP32 pipes, 7.2 ms here;
+// 16 x 16 3.46 and 1.58 ms; complex128 x complex64 16 x 32 4.93 and 2.21 ms.
+// (64-bit integer sums of one unit per column, with one conversion per digit
+// group, took 6.65, 1.51 and 2.10 ms, but were off by 2e-11 of sum |a||b| for
+// powers (4, -4) and by 1.9e-13 beside one large entry.)
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -48,6 +61,7 @@
 #include <type_traits>
 
 #include "cx.cuh"
+#include "dfloat.cuh"
 #include "pcx_internal.h"
 #include "stream_scratch.h"
 
@@ -59,11 +73,8 @@ constexpr int MAXC = 48;               // columns of A or B per launch
 constexpr int NS = 5;                  // digits
 constexpr int DB = 10;                 // bits per digit
 constexpr int MB = DB - 1 + DB * (NS - 1);   // magnitude bits of the fixed-point value
-// digit group 0 has weight 2^SUM_BITS in the 64-bit sums: the last group sits
-// 10 bits below the unit and is rounded into it, so that MAX_ROWS rows cannot
-// overflow
-constexpr int SUM_BITS = DB * (NS - 2);
-constexpr long long MAX_ROWS = 16000;  // rows per CTA: 500 chunks of at most 2^53 keep the 64-bit sums in range
+constexpr int UNIT_BITS = 2 * (DB - 1);   // a product of leading digits has the unit 2^(Ea + Eb - UNIT_BITS)
+constexpr long long MAX_ROWS = 16000;  // rows per CTA: longer columns take more waves
 constexpr int E_MIN = 128;             // smallest exponent of a complex128 column (biased): keeps 2^(MB - E) finite
 
 template <typename T>
@@ -191,6 +202,21 @@ template <int N>
 __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "n"(N) : "memory"); }
 constexpr int BAR_FULL = 1, BAR_EMPTY = 3;   // + digit buffer
 
+// v += sigma (g[0] + 2^-10 g[1] + ... + 2^-40 g[4]), the digit groups of a
+// chunk.  The first three groups are added without error (their sums are
+// integers of a few more than 24 bits; what a step rounds off the next one
+// takes up), the last two round 2^-24 of what is left; sigma is a power of
+// two.  So a chunk's sum carries 2^-48 of itself into the running TwoSum.
+using dfloat::DF;
+__device__ __forceinline__ void add_chunk(DF& v, const float g[NS], float sigma) {
+  constexpr float U1 = 1.f / (1 << DB), U2 = U1 * U1, U3 = U2 * U1;
+  const float p = fmaf(g[1], U1, g[0]);
+  const float q = fmaf(g[2], U2, fmaf(g[1], U1, -__fsub_rn(p, g[0])));
+  const float h = __fadd_rn(p, q);
+  const float l = fmaf(fmaf(g[4], U1, g[3]), U3, __fsub_rn(q, __fsub_rn(h, p)));
+  dfloat::add(v, __fmul_rn(h, sigma), __fmul_rn(l, sigma));
+}
+
 __device__ __forceinline__ void mma16816_zero(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};\n"
@@ -230,12 +256,16 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
   int* expo = reinterpret_cast<int*>(raw + 2 * raw_bytes);           // [3][2 MAXC]
   int* changed = expo + 3 * 2 * MAXC;                                // [3]
   int* bad = changed + 4;                                            // [2 MAXC]
+  float* ratio = reinterpret_cast<float*>(bad + 2 * MAXC);           // [2][2 MAXC]: 2^(chunk's exponent - running one)
   for (int i = tid; i < 2 * buf_bytes / 16; i += THREADS) reinterpret_cast<uint4*>(sm)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < 3 * 2 * MAXC; i += THREADS) {
     const bool dbl = i % (2 * MAXC) < MAXC ? sizeof(TA) == 8 : sizeof(TB) == 8;
     expo[i] = dbl ? E_MIN : 1;
   }
-  for (int i = tid; i < 2 * MAXC; i += THREADS) bad[i] = 0;
+  for (int i = tid; i < 2 * MAXC; i += THREADS) {
+    bad[i] = 0;
+    ratio[i] = ratio[2 * MAXC + i] = 0.f;
+  }
   if (tid < 4) changed[tid] = 0;
   __syncthreads();
 
@@ -273,7 +303,8 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
       using C = std::remove_const_t<std::remove_pointer_t<decltype(entries)>>;
       using T = decltype(C::x);
       using F = Fields<T>;
-      constexpr int NB = 2;
+      constexpr int NB = 2, EMIN = sizeof(T) == 8 ? E_MIN : 1;
+      float* rt = ratio + (f & 1) * 2 * MAXC + x0;
       const int* eold = expo + ((f + 2) % 3) * 2 * MAXC + x0;
       int* enew = expo + (f % 3) * 2 * MAXC + x0;
       for (int p0 = sw; p0 < npair; p0 += NB * SW) {
@@ -297,10 +328,12 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
           const int p = p0 + b * SW, c = 2 * p + half;
           if (p >= npair) break;
           const bool isbad = E[b] == Entry<T>::BAD;
-          E[b] = max(E[b], old[b]);
+          E[b] = max(E[b], EMIN);
           if (q == 0 && c < ncol) {
-            enew[c] = E[b];
-            if (E[b] != old[b]) changed[f % 3] = 1;
+            const int top = max(E[b], old[b]);
+            enew[c] = top;
+            rt[c] = __int_as_float(max(127 + E[b] - top, 0) << 23);
+            if (top != old[b]) changed[f % 3] = 1;
             if (isbad) bad[x0 + c] = 1;
           }
           const auto sc = scale_of((T)0, E[b]);
@@ -351,7 +384,7 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
   const int tr_n = ra / 16, tc_n = rb / 16;
   const int items = g.sym ? tr_n * (tr_n + 1) / 2 : tr_n * tc_n;
   int tile[MT];   // row tile << 8 | column tile (-1: none)
-  long long v[MT][8];
+  DF v[MT][8];    // sums in units of 2^(running exponents - UNIT_BITS)
 #pragma unroll
   for (int k = 0; k < MT; ++k) {
     int it = warp + k * MW, r = 0;
@@ -371,12 +404,12 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
       tile[k] = r << 8 | it;
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[k][i] = 0;
+    for (int i = 0; i < 8; ++i) v[k][i] = DF{0.f, 0.f};
   }
   const int gid = lane >> 2, tg = lane & 3;
   // exponent slot of a real row of A / real column of B (padding: slot of column 0, their sums are 0)
-  auto slot_a = [&](int r) { const int c = r % g.na8; return c < g.na ? c : 0; };
-  auto slot_b = [&](int r) { const int c = r % g.nb8; return (g.sym ? 0 : MAXC) + (c < g.nb ? c : 0); };
+  auto slot_a = [&](int r) { const int c = r < g.na8 ? r : r - g.na8; return c < g.na ? c : 0; };
+  auto slot_b = [&](int r) { const int c = r < g.nb8 ? r : r - g.nb8; return (g.sym ? 0 : MAXC) + (c < g.nb ? c : 0); };
 
   for (int f = 0; f < nch; ++f) {
     bar_wait<THREADS>(BAR_FULL + (f & 1));
@@ -395,7 +428,9 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
           const int sa = slot_a(tr * 16 + gid + 8 * ((i >> 1) & 1));
           const int sb = slot_b(tc * 16 + 8 * (i >> 2) + 2 * tg + (i & 1));
           const int sh = (e1[sa] - e0[sa]) + (e1[sb] - e0[sb]);
-          v[k][i] >>= sh > 63 ? 63 : sh;
+          const float w = __int_as_float(max(127 - sh, 0) << 23);
+          v[k][i].s *= w;
+          v[k][i].c *= w;
         }
       }
       float acc[NS][8];
@@ -424,18 +459,18 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
           }
         }
       }
-      // the chunk's exact sums into the 64-bit sums
+      // the chunk's sums join the running ones
+      const float* rt = ratio + (f & 1) * 2 * MAXC;
+      float ra2[2], rb4[4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) ra2[i] = rt[slot_a(tr * 16 + gid + 8 * i)];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rb4[i] = rt[slot_b(tc * 16 + 8 * (i >> 1) + 2 * tg + (i & 1))];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        long long t = v[k][i];
-#pragma unroll
-        for (int w = 0; w < NS - 1; ++w) {
-          // the unit of the 64-bit sums is that of group 3: the last of five
-          // groups joins it as a fraction and is rounded with it
-          const float xf = w == NS - 2 ? fmaf(acc[NS - 1][i], 1.f / (float)(1 << DB), acc[w][i]) : acc[w][i];
-          t += (long long)__float2int_rn(xf) * (1ll << (SUM_BITS - DB * w));
-        }
-        v[k][i] = t;
+        const float g5[NS] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i], acc[4][i]};
+        add_chunk(v[k][i], g5, ra2[(i >> 1) & 1] * rb4[2 * (i >> 2) + (i & 1)]);
+        if ((f & 3) == 3) dfloat::renorm(v[k][i]);
       }
     }
     if (f + 2 < nch) bar_arrive<THREADS>(BAR_EMPTY + (f & 1));
@@ -450,8 +485,8 @@ __global__ void __launch_bounds__((MW + SW) * 32, CTAS) gram_digits_kernel(Digit
     for (int i = 0; i < 8; ++i) {
       const int r = tr * 16 + gid + 8 * ((i >> 1) & 1), c = tc * 16 + 8 * (i >> 2) + 2 * tg + (i & 1);
       const int sa = slot_a(r), sb = slot_b(c);
-      double d = ldexp((double)v[k][i], expo[ef + sa] - Entry<TA>::BIAS + expo[ef + sb] - Entry<TB>::BIAS -
-                                            (SUM_BITS + 2 * (DB - 1)));
+      double d = ldexp((double)v[k][i].s + (double)v[k][i].c,
+                       expo[ef + sa] - Entry<TA>::BIAS + expo[ef + sb] - Entry<TB>::BIAS - UNIT_BITS);
       if (bad[sa] | bad[sb]) d = __longlong_as_double(0x7ff8000000000000LL);
       out[(size_t)r * rb + c] = d;
     }
@@ -514,7 +549,7 @@ cudaError_t run_block(DigitArgs g, int sms, double* G, int ldg, cudaStream_t s) 
   const int rtot = 2 * g.na8 + (g.sym ? 0 : 2 * g.nb8);
   const size_t smem = (size_t)2 * NS * rtot * 64 + (size_t)2 * ((g.na + 1) / 2) * 64 * sizeof(typename Entry<TA>::C) +
                       (g.sym ? 0 : (size_t)2 * ((g.nb + 1) / 2) * 64 * sizeof(typename Entry<TB>::C)) +
-                      (3 * 2 * MAXC + 4 + 2 * MAXC) * sizeof(int);
+                      (3 * 2 * MAXC + 4 + 2 * MAXC) * sizeof(int) + 2 * 2 * MAXC * sizeof(float);
   cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   if constexpr (REG > 0) {

@@ -133,3 +133,53 @@ def test_long_columns(pcx):
     v = L * (1.0 - 2.0 ** -52) ** 2
     want = np.array([[v, -1j * v], [1j * v, v]])
     assert np.abs(G.cpu().numpy() - want).max() <= v * 2.0 ** -44
+
+
+# Columns graded against each other and columns with one dominant entry.
+#
+# An entry is cut relative to its column's largest part M_c in its chunk of 32
+# rows (2^E <= 2 M_c).  The pairs left out and the rounding of the entries come
+# to 2^-50 2^(Ea + Eb) rms in a real product, so 2^-47.5 sqrt(sum over rows of
+# (M_c M'_c)^2) in an entry of G; the tolerance takes 11 times that.  The sums
+# of the chunks are kept to about 2^-49 of the running sum at each addition:
+# 2^-47 sum |a||b| holds for them with room.
+def _graded_bound(a, b):
+    L = a.shape[1]
+    mag = [np.maximum(np.abs(v.real), np.abs(v.imag)).reshape(v.shape[0], L // 32, 32).max(axis=2) for v in (a, b)]
+    sq = 32 * (mag[0] ** 2 @ (mag[1] ** 2).T)
+    return 2.0 ** -44 * np.sqrt(sq) + 2.0 ** -47 * (np.abs(a) @ np.abs(b).T.astype(np.float64))
+
+
+@pytest.mark.parametrize("decades", [3, 6, 9])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("na,nb", [(2, 3), (18, 17), (35, 3)])
+def test_graded_columns(pcx, decades, mixed, na, nb):
+    """A falls and B rises by `decades` over every 1024 rows, so all rows weigh alike in the products."""
+    L = 32 * 6250
+    t = 10.0 ** (decades * (np.arange(L) % 1024) / 1024.0)
+    rng = np.random.default_rng(decades)
+    cx = lambda *sh: rng.standard_normal(sh) + 1j * rng.standard_normal(sh)
+    a = cx(na, L) / t
+    b = (cx(nb, L) * t).astype(np.complex64 if mixed else np.complex128)
+    got = _gram(pcx, a, b)
+    want = np.zeros((na, nb), dtype=np.clongdouble)
+    for i in range(na):
+        for j in range(nb):
+            want[i, j] = (a[i].conj().astype(np.clongdouble) * b[j].astype(np.clongdouble)).sum()
+    assert np.all(np.abs(got - want) <= _graded_bound(a, b))
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_dominant_entry(pcx, mixed):
+    """One entry 1000 times the others in long columns.  Its chunk errs by about 2^-47 M M' (as above); the other
+    chunks are cut by their own size, and adding some hundred of them to the large sum costs 2^-45.5 M M' at most
+    where all roundings add up as a random walk: 2^-43 M M' in all."""
+    L = 2 * 10 ** 6
+    rng = np.random.default_rng(11)
+    cx = lambda *sh: rng.standard_normal(sh) + 1j * rng.standard_normal(sh)
+    a, b = cx(2, L), cx(2, L)
+    a[:, 5], b[:, 5] = 1000.0 - 300.0j, 700.0 + 900.0j
+    b = b.astype(np.complex64 if mixed else np.complex128)
+    got = _gram(pcx, a, b)
+    want = np.array([[(x.conj().astype(np.clongdouble) * y.astype(np.clongdouble)).sum() for y in b] for x in a])
+    assert np.abs(got - want).max() <= 2.0 ** -43 * 1000.0 * 900.0
