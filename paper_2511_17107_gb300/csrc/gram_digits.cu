@@ -552,16 +552,6 @@ cudaError_t run_block(DigitArgs g, int sms, double* G, int ldg, cudaStream_t s) 
                       (3 * 2 * MAXC + 4 + 2 * MAXC) * sizeof(int) + 2 * 2 * MAXC * sizeof(float);
   cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  if constexpr (REG > 0) {
-    // the split hands out what the launch allocated: it must be 128 a thread
-    static std::atomic<int> regs{0};
-    if (regs.load() == 0) {
-      cudaFuncAttributes fa;
-      if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-      regs.store(fa.numRegs);
-    }
-    if (regs.load() != 128) return cudaErrorInvalidConfiguration;
-  }
   // whole waves of CTAs, at least 4 chunks and at most MAX_ROWS rows each
   const long long chunks = (g.L + KC - 1) / KC;
   const long long fill = (long long)CTAS * sms;
@@ -581,14 +571,39 @@ cudaError_t run_block(DigitArgs g, int sms, double* G, int ldg, cudaStream_t s) 
   return cudaGetLastError();
 }
 
+// Whether the kernels of the wide products may run: their register split hands
+// out what the launch allocated, so the compiler must have given them exactly
+// 128 registers a thread (it does, at the launch bounds' limit).
+template <typename TA, typename TB>
+cudaError_t wide_kernels(bool* ok) {
+  static std::atomic<int> state{0};   // 1: yes, 2: no
+  if (state.load() == 0) {
+    bool all = true;
+    for (auto kern : {gram_digits_kernel<TA, TB, 8, 8, 2, 1, 144>, gram_digits_kernel<TA, TB, 8, 8, 3, 1, 152>,
+                      gram_digits_kernel<TA, TB, 8, 8, 5, 1, 184>}) {
+      cudaFuncAttributes fa;
+      const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+      if (e != cudaSuccess) return e;
+      all = all && fa.numRegs == 128;
+    }
+    state.store(all ? 1 : 2);
+  }
+  *ok = state.load() == 1;
+  return cudaSuccess;
+}
+
 template <typename TA, typename TB>
 cudaError_t run_digits(const void* A, int na, const void* B, int nb, size_t L, double* G, cudaStream_t s) {
   int dev = 0, sms = 0;
+  bool wide = true;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = wide_kernels<TA, TB>(&wide);
   if (e != cudaSuccess) return e;
-  // column blocks of at most MAXC
-  const int ba = (na + MAXC - 1) / MAXC, bb = (nb + MAXC - 1) / MAXC;
+  // column blocks of at most MAXC, or of what the kernels without a register
+  // split take (8 tiles)
+  const int ca = wide ? MAXC : 16, cb = wide ? MAXC : 32;
+  const int ba = (na + ca - 1) / ca, bb = (nb + cb - 1) / cb;
   const int sa = (na + ba - 1) / ba, sb = (nb + bb - 1) / bb;
   for (int i0 = 0; i0 < na; i0 += sa)
     for (int j0 = 0; j0 < nb; j0 += sb) {
