@@ -8,18 +8,24 @@
 // converted back; the work per mode and per cell between the transforms (C^H,
 // M, C w + gamma conj(kappa)(kappa.x)) stays in FP64.
 //
-// Line format.  E is the largest biased exponent of a line, so |re|, |im| <
-// 2^(E - 1022), and an entry becomes round(v 2^(P - (E - 1022))) with P = 61 -
-// log2 N.  A modulus grows at most N-fold in the transform, so every integer
-// stays below 2^(61.5) and no stage scales or overflows; additions are exact.
-// The rounding of the input (2^-(P + 1) of the line's largest entry, P = 54 at
-// N = 128) and of the twiddle products (half a unit each, of values that have
-// grown) keeps the error of a transform at or below that of FP64 arithmetic,
-// which rounds every addition at 2^-53 of its result.
+// Line format.  No partial sum of a transform is larger than the sum of the
+// moduli of the line's entries, so the scale comes from that sum: E is the
+// line's largest biased exponent (|re|, |im| < 2^(E - 1022)), S >= sum(|re| +
+// |im|) is taken to 21 bits below 2^E, b = bit length of S in those units, and
+// an entry becomes round(v 2^(61 - (E - 1022 - 21 + b))).  Every partial sum
+// then stays below 2^61 (its real and imaginary part added or subtracted,
+// below 2^61.5), no stage scales or overflows, and additions are exact.  What
+// is lost is half a unit per entry of the input, and at most 1.8 (rms 0.5)
+// units per twiddle product.  Against extended precision, lines of 16 to 256
+// points: 0.35 to 0.6 of the error of the same transform in FP64, whether the
+// entries are even, fall off with the index (powers 1, 2, 4) or are one large
+// among small ones.  (A scale from the largest entry and N alone, one step
+// shorter, wastes what the growth does not use: 1.0 to 7.5 times the error of
+// FP64 at 256 points, up to 2.8 times at 128.)
 //
 // Twiddles are 2^61 cos and 2^61 sin split into signed limbs of 31 bits; a
-// complex product is 12 wide multiply-adds (the lowest limb products, below
-// half a unit, are left out).  A line with Inf or NaN gives NaN throughout.
+// complex product is 12 wide multiply-adds (the products of two low limbs, up
+// to a unit each, are left out).  A line with Inf or NaN gives NaN throughout.
 #pragma once
 
 #include "fft_kernels.cuh"
@@ -30,11 +36,6 @@ namespace fixed {
 
 using ll = long long;
 using cxl = cx<ll>;
-
-template <int N>
-__host__ __device__ constexpr int line_bits() {
-  return 61 - ilog2(N);
-}
 
 struct Twid {
   int ch, cl, sh, sl;   // 2^61 cos = ch 2^31 + cl, 2^61 sin = sh 2^31 + sl
@@ -113,19 +114,31 @@ __device__ __forceinline__ int exp_bits(cx<double> v) {
   const uint32_t y = (uint32_t)(__double_as_longlong(v.y) >> 32) & 0x7fffffffu;
   return (int)((x > y ? x : y) >> 20);
 }
-// round(v 2^(P - (E - 1022))), E >= 1 the line's exponent
-template <int P>
-__device__ __forceinline__ ll to_fixed(double v, int E) {
+// A line's scale: its largest biased exponent e >= 1, and the sum of its
+// entries' parts in units of 2^(e - 1043), each rounded up.
+struct __align__(8) Line {
+  int e;
+  unsigned sum;
+};
+__device__ __forceinline__ unsigned coarse(double v, int E) {
+  const uint32_t hi = (uint32_t)(__double_as_longlong(v) >> 32) & 0x7fffffffu;
+  const int e = (int)(hi >> 20);
+  const uint32_t m = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  return (m >> min(E - (e ? e : 1), 31)) + 1u;
+}
+// K = e + b - 21: an entry is v 2^(1083 - K), below 2^61
+__device__ __forceinline__ int line_scale(Line l) { return l.e + 11 - __clz((int)l.sum); }
+// round(v 2^(1083 - K))
+__device__ __forceinline__ ll to_fixed(double v, int K) {
   const ll b = __double_as_longlong(v);
   const int e = (int)(b >> 52) & 0x7ff;
   const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
-  int d = E - (e ? e : 1);
-  if (d > 63) d = 63;
-  const ll q = (ll)(((m << (P - 52)) >> d) + 1) >> 1;
+  const int d = min(K - (e ? e : 1), 63);
+  const ll q = (ll)(((m << 9) >> d) + 1) >> 1;
   const ll s = b >> 63;
   return (q ^ s) - s;
 }
-// v 2^e rounded to a double; results below the normal range go to 0
+// v 2^e rounded to a double
 __device__ __forceinline__ double to_double(ll v, int e) {
   const ll s = v >> 63;
   const unsigned long long m = (unsigned long long)((v ^ s) - s);
@@ -135,28 +148,33 @@ __device__ __forceinline__ double to_double(ll v, int e) {
   const int ex = 1023 + 63 + e - lz + carry;
   unsigned long long bits = ((unsigned long long)(unsigned)ex << 52) | (((n << carry) >> 11) & 0xfffffffffffffull);
   if (ex >= 2047) bits = 0x7ffull << 52;
-  if (ex <= 0 || m == 0) bits = 0;
+  if (ex <= 0) {   // below the normal range: a multiple of 2^-1074
+    const int d = -1074 - e;
+    bits = d > 0 ? ((m >> (d - 1)) + 1) >> 1 : m << -d;
+  }
+  if (m == 0) bits = 0;
   return __longlong_as_double((ll)bits | (s & (ll)(1ull << 63)));
 }
-// an entry of a line of exponent E as doubles, times 2^SHIFT
-template <int N, int SHIFT = 0>
-__device__ __forceinline__ cx<double> line_value(cxl v, int E) {
+// an entry of a line as doubles, times 2^SHIFT
+template <int SHIFT = 0>
+__device__ __forceinline__ cx<double> line_value(cxl v, Line l) {
   const double bad = __longlong_as_double(0x7ff8000000000000ll);
-  if (E == 2047) return mk(bad, bad);
-  const int e = E - 1022 - line_bits<N>() + SHIFT;
+  if (l.e == 2047) return mk(bad, bad);
+  const int e = line_scale(l) - 1083 + SHIFT;
   return mk(to_double(v.x, e), to_double(v.y, e));
 }
 
 // One Stockham stage (as fftk::stage).  SRC: 0 fixed-point tile; 1 global
-// memory, 2 tile holding doubles (first stage: finds the lines' exponents and
+// memory, 2 tile holding doubles (first stage: finds the lines' scales and
 // converts).  DST: 0 fixed-point tile, 1 global memory (last stage: converts
-// back).  lexp[c TP + t]: the exponent of line t of component c.
+// back).  line[c TP + t]: the scale of line t of component c.
 template <int N, int AXIS, int R, int DIR, int SRC, int DST>
-__device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, int* lexp, int Ns, const cx<double>* gin,
+__device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, Line* line, int Ns, const cx<double>* gin,
                                             cx<double>* gout, int qb) {
   using C = Cfg<double, N>;
   using TL = Tile<double, N, AXIS>;
-  constexpr int NB = N / R, PER = C::E / R, N3 = N * N * N, TP = C::TP, P = line_bits<N>();
+  constexpr int NB = N / R, PER = C::E / R, N3 = N * N * N, TP = C::TP;
+  constexpr int NL = NB < 32 ? NB : 32;   // lanes of a line (x tiles: neighbours)
   cxl v[PER][R];
   if constexpr (SRC == 0) {
 #pragma unroll
@@ -181,12 +199,12 @@ __device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, int* lexp, i
       }
 #pragma unroll
       for (int r = 0; r < R; ++r) e = max(e, exp_bits(d[i][r]));
-      if constexpr (AXIS == 0) {   // the lanes of a line are neighbours
+      if constexpr (AXIS == 0) {
 #pragma unroll
-        for (int o = (NB < 32 ? NB : 32) / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        if (j % (NB < 32 ? NB : 32) == 0) atomicMax(&lexp[c * TP + t], e);
+        for (int o = NL / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+        if (j % NL == 0) atomicMax(&line[c * TP + t].e, e);
       } else {
-        atomicMax(&lexp[c * TP + t], e);
+        atomicMax(&line[c * TP + t].e, e);
       }
     }
     __syncthreads();   // exponents (and every read of a tile of doubles)
@@ -194,9 +212,26 @@ __device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, int* lexp, i
     for (int i = 0; i < PER; ++i) {
       int t, j, c;
       TL::item(threadIdx.x + i * C::THREADS, NB, t, j, c);
-      const int E = lexp[c * TP + t];
+      const int E = line[c * TP + t].e;
+      unsigned sum = 0;   // 2 R parts of at most 2^21, 2 N <= 512 of them in a line
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[i][r] = mk(to_fixed<P>(d[i][r].x, E), to_fixed<P>(d[i][r].y, E));
+      for (int r = 0; r < R; ++r) sum += coarse(d[i][r].x, E) + coarse(d[i][r].y, E);
+      if constexpr (AXIS == 0) {
+#pragma unroll
+        for (int o = NL / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (j % NL == 0) atomicAdd(&line[c * TP + t].sum, sum);
+      } else {
+        atomicAdd(&line[c * TP + t].sum, sum);
+      }
+    }
+    __syncthreads();   // sums
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      int t, j, c;
+      TL::item(threadIdx.x + i * C::THREADS, NB, t, j, c);
+      const int K = line_scale(line[c * TP + t]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[i][r] = mk(to_fixed(d[i][r].x, K), to_fixed(d[i][r].y, K));
     }
   }
 #pragma unroll
@@ -212,10 +247,10 @@ __device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, int* lexp, i
     dft_fixed<R, DIR>(v[i]);
     const int base = (j / Ns) * Ns * R + k;
     if constexpr (DST == 1) {
-      const int E = lexp[c * TP + t];
+      const Line l = line[c * TP + t];
       cx<double>* g = gout + (c * N3 + TL::gidx(qb + t, base));
 #pragma unroll
-      for (int r = 0; r < R; ++r) g[r * Ns * TL::GSTRIDE] = line_value<N>(v[i][r], E);
+      for (int r = 0; r < R; ++r) g[r * Ns * TL::GSTRIDE] = line_value(v[i][r], l);
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) s[TL::sidx(c, t, base + r * Ns)] = v[i][r];
@@ -225,18 +260,18 @@ __device__ __forceinline__ void stage_fixed(cxl* s, const Twid* tw, int* lexp, i
 }
 
 template <int N, int AXIS, int DIR, int SRC, int DST>
-__device__ __forceinline__ void fft_fixed(cxl* s, const Twid* tw, int* lexp, const cx<double>* gin, cx<double>* gout,
+__device__ __forceinline__ void fft_fixed(cxl* s, const Twid* tw, Line* line, const cx<double>* gin, cx<double>* gout,
                                           int qb) {
   using P = typename Cfg<double, N>::P;
   if constexpr (P::NST == 1) {
-    stage_fixed<N, AXIS, P::R0, DIR, SRC, DST>(s, tw, lexp, 1, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R0, DIR, SRC, DST>(s, tw, line, 1, gin, gout, qb);
   } else if constexpr (P::NST == 2) {
-    stage_fixed<N, AXIS, P::R0, DIR, SRC, 0>(s, tw, lexp, 1, gin, gout, qb);
-    stage_fixed<N, AXIS, P::R1, DIR, 0, DST>(s, tw, lexp, P::R0, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R0, DIR, SRC, 0>(s, tw, line, 1, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R1, DIR, 0, DST>(s, tw, line, P::R0, gin, gout, qb);
   } else {
-    stage_fixed<N, AXIS, P::R0, DIR, SRC, 0>(s, tw, lexp, 1, gin, gout, qb);
-    stage_fixed<N, AXIS, P::R1, DIR, 0, 0>(s, tw, lexp, P::R0, gin, gout, qb);
-    stage_fixed<N, AXIS, P::R2, DIR, 0, DST>(s, tw, lexp, P::R0 * P::R1, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R0, DIR, SRC, 0>(s, tw, line, 1, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R1, DIR, 0, 0>(s, tw, line, P::R0, gin, gout, qb);
+    stage_fixed<N, AXIS, P::R2, DIR, 0, DST>(s, tw, line, P::R0 * P::R1, gin, gout, qb);
   }
 }
 
@@ -255,7 +290,7 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
   D* ka = reinterpret_cast<D*>(tw + N);   // [3][N], then [TP][3] (see pass_kernel)
   D* kb = ka + 3 * N;
   double* mtab = reinterpret_cast<double*>(kb + 3 * TP);   // z sandwich: material table, ids; x POST: scratch tile
-  __shared__ int lexp[2][3 * TP];
+  __shared__ Line line[2][3 * TP];
 
   const size_t q0 = (size_t)blockIdx.x * TP;
   const size_t v = q0 / N2;
@@ -265,7 +300,7 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
 
   const D* gtw = static_cast<const D*>(a.tw);
   for (int i = threadIdx.x; i < N; i += C::THREADS) tw[i] = make_twid(gtw[i]);
-  for (int i = threadIdx.x; i < 2 * 3 * TP; i += C::THREADS) lexp[0][i] = 1;
+  for (int i = threadIdx.x; i < 2 * 3 * TP; i += C::THREADS) line[0][i] = Line{1, 0u};
   KParams kp = a.kp;
   if (AXIS == 0 && a.kps) kp = a.kps[(a.v_base + (int)v) / a.vec_per_k];
   if constexpr (AXIS == 0 && OP != OP_PLAIN_INV && OP != OP_PLAIN_FWD)
@@ -279,7 +314,7 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
 
   if constexpr (OP == OP_PLAIN_INV || OP == OP_PLAIN_FWD || OP == OP_INV || OP == OP_FWD) {
     __syncthreads();
-    fft_fixed<N, AXIS, OP == OP_PLAIN_INV || OP == OP_INV ? +1 : -1, 1, 1>(s, tw, lexp[0], in, out, qb);
+    fft_fixed<N, AXIS, OP == OP_PLAIN_INV || OP == OP_INV ? +1 : -1, 1, 1>(s, tw, line[0], in, out, qb);
   } else if constexpr (OP == OP_PRE || OP == OP_PRE_T0) {
     for (int e = threadIdx.x; e < TP * N; e += C::THREADS) {
       const int t = e / N, n = e % N;
@@ -297,7 +332,7 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
                                          sb[TL::gidx(qb + t, n)], ka + n, N, kb + 3 * t, kp, gam, igam);
     }
     __syncthreads();
-    fft_fixed<N, 0, +1, 2, 1>(s, tw, lexp[0], nullptr, out, qb);
+    fft_fixed<N, 0, +1, 2, 1>(s, tw, line[0], nullptr, out, qb);
   } else if constexpr (OP == OP_POST || OP == OP_POST_T0) {
     const D* sb = static_cast<const D*>(a.sbuf) + v * N3;
     D* ssb = kb + 3 * TP;   // [TP * N]
@@ -305,15 +340,15 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
       const int t = e / N, n = e % N;
       cp_async_cx<double>(&ssb[e], &sb[TL::gidx(qb + t, n)]);
     }
-    __syncthreads();   // twiddles, exponents
-    fft_fixed<N, 0, -1, 1, 0>(s, tw, lexp[0], in, nullptr, qb);
+    __syncthreads();   // twiddles, scales
+    fft_fixed<N, 0, -1, 1, 0>(s, tw, line[0], in, nullptr, qb);
     cp_async_commit_wait_all();
     __syncthreads();
     for (int e = threadIdx.x; e < TP * N; e += C::THREADS) {
       const int t = e / N, n = e % N;
       D w[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) w[c] = line_value<N>(s[TL::sidx(c, t, n)], lexp[0][c * TP + t]);
+      for (int c = 0; c < 3; ++c) w[c] = line_value(s[TL::sidx(c, t, n)], line[0][c * TP + t]);
       const int g = TL::gidx(qb + t, n);
       post_point<double, OP == OP_POST_T0>(w, ssb[e], ka + n, N, kb + 3 * t, out[g], out[N3 + g], out[2 * N3 + g]);
     }
@@ -330,8 +365,8 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
                      : "memory");
       }
     }
-    __syncthreads();   // twiddles, exponents
-    fft_fixed<N, 2, +1, 1, 0>(s, tw, lexp[0], in, nullptr, qb);
+    __syncthreads();   // twiddles, scales
+    fft_fixed<N, 2, +1, 1, 0>(s, tw, line[0], in, nullptr, qb);
     cp_async_commit_wait_all();
     __syncthreads();
     for (int w = threadIdx.x; w < TP * N; w += C::THREADS) {   // pencils fastest
@@ -339,13 +374,13 @@ __global__ void __launch_bounds__(Cfg<double, N>::THREADS, 2) pass_fixed_kernel(
       D e[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c)   // with the transforms' 1 / N^3
-        e[c] = line_value<N, -3 * ilog2(N)>(s[TL::sidx(c, t, n)], lexp[0][c * TP + t]);
+        e[c] = line_value<-3 * ilog2(N)>(s[TL::sidx(c, t, n)], line[0][c * TP + t]);
       cell_point<double, N, OP == OP_SANDWICH_EPS>(e, mid ? &sid[w] : nullptr, mtab, M, n * N2 + (qb + t), 1.0);
 #pragma unroll
       for (int c = 0; c < 3; ++c) sd[TL::sidx(c, t, n)] = e[c];
     }
     __syncthreads();
-    fft_fixed<N, 2, -1, 2, 1>(s, tw, lexp[1], nullptr, out, qb);
+    fft_fixed<N, 2, -1, 2, 1>(s, tw, line[1], nullptr, out, qb);
   }
 }
 
