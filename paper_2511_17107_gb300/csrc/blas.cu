@@ -372,6 +372,24 @@ __global__ void __launch_bounds__(256) combine_add32_kernel(const cx<float>* __r
   }
 }
 
+// A few FP32 squares as a double-float pair.  A square that takes the pair
+// beyond the FP32 range (or is Inf or NaN itself) goes to the FP64 sum alone,
+// so the sum has the range of FP64 and infinities stay infinite.
+struct SquareSum {
+  dfloat::DF p{0.f, 0.f};
+  __device__ __forceinline__ void add(float q, double& total) {
+    if (!(__fadd_rn(p.s, q) <= 3.402823466e38f)) {
+      total += (double)q;
+      return;
+    }
+    dfloat::add(p, q, 0.f);
+  }
+  __device__ __forceinline__ void flush(double& total) {
+    total += (double)p.s + (double)p.c;
+    p = dfloat::DF{0.f, 0.f};
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Residual R_j = AX_j - theta_j X_j with ||R_j||^2 and ||X_j||^2 (FP64).
 // ---------------------------------------------------------------------------
@@ -380,11 +398,13 @@ __global__ void __launch_bounds__(256) residual_kernel(const cx<T>* __restrict__
                                                        cx<T>* R, double* norms, int nvec, size_t L) {
   const int j = blockIdx.y;
   const T th = (T)theta[j];
-  // squares summed per thread in FP64 (complex128) or as double-float pairs on
-  // the FP32 pipes (complex64: two FP64 conversions and additions per entry
-  // bound the kernel at 0.80 ms for 16 columns of 3 128^3, 0.39 ms so)
+  // squares summed per thread in FP64.  complex64: two FP64 conversions and
+  // additions per entry bound the kernel at 0.80 ms for 16 columns of 3 128^3;
+  // so eight squares gather in a double-float pair on the FP32 pipes before
+  // they are added (the pair rounds at 2^-48, each FP32 square at 2^-24).
   double rr = 0.0, xx = 0.0;
-  dfloat::DF rf{0.f, 0.f}, xf{0.f, 0.f};
+  SquareSum rf, xf;
+  int pending = 0;
   const cx<T>* x = X + (size_t)j * L;
   const cx<T>* ax = AX + (size_t)j * L;
   cx<T>* r = R + (size_t)j * L;
@@ -393,16 +413,21 @@ __global__ void __launch_bounds__(256) residual_kernel(const cx<T>* __restrict__
     const cx<T> rv = mk(fma(-th, xv.x, av.x), fma(-th, xv.y, av.y));
     r[l] = rv;
     if constexpr (sizeof(T) == 4) {
-      dfloat::add(rf, norm2(rv), 0.f);
-      dfloat::add(xf, norm2(xv), 0.f);
+      rf.add(norm2(rv), rr);
+      xf.add(norm2(xv), xx);
+      if (++pending == 8) {
+        rf.flush(rr);
+        xf.flush(xx);
+        pending = 0;
+      }
     } else {
       rr = fma(rv.x, rv.x, fma(rv.y, rv.y, rr));
       xx = fma(xv.x, xv.x, fma(xv.y, xv.y, xx));
     }
   }
   if constexpr (sizeof(T) == 4) {
-    rr = (double)rf.s + (double)rf.c;
-    xx = (double)xf.s + (double)xf.c;
+    rf.flush(rr);
+    xf.flush(xx);
   }
   __shared__ double red[2][32];
   for (int o = 16; o > 0; o >>= 1) {
