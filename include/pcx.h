@@ -208,7 +208,7 @@ pcx_status pcx_symbols(const pcx_ctx* ctx, const double k[3], double gamma,
  * vectors that run through all FFT passes before the next ones start (a block
  * is split into launches of equal size).  chunk <= 0 restores the default:
  * as many vectors as 256 MiB of scratch hold (one at least), or for
- * M_CrossDoF a single vector where half of L2 holds no more.
+ * M_CrossDoF in complex64 as many as half of L2 holds.
  * Host-only; affects calls issued afterwards.
  */
 pcx_status pcx_set_apply_chunk(pcx_ctx* ctx, int chunk);

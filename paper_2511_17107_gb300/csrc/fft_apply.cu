@@ -54,17 +54,19 @@ cudaError_t dispatch_apply(const pcx_ctx* c, const KParams& kp, const void* X, v
 // 109.7 us, 16 take 99.1 us each; at 64^3, 13 vectors in one launch 13.9 us
 // each, 10 and 3 14.7 us; in complex128 at 128^3 836 against 774 us.  So a
 // chunk is as many vectors as a scratch of 256 MiB holds.  The M_CrossDoF
-// chain keeps one vector per launch where that is what half of L2 holds (its
-// stencil pass reads every value 9 times: 173 us at 128^3 against 177), and a
-// context whose scratch could not be allocated stays with what half of L2
-// holds.
+// chain of complex64 stays with what half of L2 holds, its stencil pass reads
+// every value 9 times (128^3, four vectors one by one 697 us, in one launch 736;
+// 64^3, 24 vectors in launches of 8 478 us, in one 491); that of complex128,
+// bound by the FP64 pipe, gains by groups (64^3, 24 vectors 3.34 ms in launches
+// of 12, 3.92 in launches of 5).  A context whose scratch could not be allocated
+// stays with what half of L2 holds.
 int apply_chunk(const pcx_ctx* c, int precision) {
   if (c->apply_chunk > 0) return c->apply_chunk;
   const size_t es = precision == PCX_FP64 ? 16 : 8, n3 = (size_t)c->n * c->n * c->n;
   const size_t l2 = c->l2_bytes ? c->l2_bytes : ((size_t)126 << 20);
   const size_t k = (l2 / 2) / (3 * n3 * es);
   const bool cross = c->m_kind == PCX_M_CROSSDOF;
-  if (c->small_scratch || (cross && k <= 1)) return (int)(k < 1 ? 1 : (k > 64 ? 64 : k));
+  if (c->small_scratch || (cross && precision == PCX_FP32)) return (int)(k < 1 ? 1 : (k > 64 ? 64 : k));
   const size_t fit = ((size_t)256 << 20) / (n3 * es * (cross ? 4 : 1));
   return (int)(fit < 1 ? 1 : (fit > 4096 ? 4096 : fit));
 }

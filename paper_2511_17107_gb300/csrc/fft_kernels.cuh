@@ -836,51 +836,80 @@ __global__ void eps_cells_kernel(const cx<T>* E, const cx<T>* __restrict__ Add, 
 //   sum over the four points q of (e_ij at E_i of the cell + e_ij at E_j of q) / 8 E^j[q],
 // one complex coefficient per neighbour, and the same for block (j, i).
 //
+template <typename T>
+struct CrossStencil {
+  // block b: component row(b) from component col(b); pair, and the offset
+  // (d = 0, 1, 2: dz, dy, dx) of its four points k: (i, j) of each pair, then (j, i)
+  static __device__ __forceinline__ int row(int b) { return b >> 1; }
+  static __device__ __forceinline__ int col(int b) {
+    constexpr int t[6] = {1, 2, 2, 0, 0, 1};
+    return t[b];
+  }
+  static __device__ __forceinline__ int pair(int b) { return b % 3; }
+  static __device__ __forceinline__ int ofs(int b, int k, int d) {
+    constexpr int t[6][4][3] = {{{0, 0, 0}, {0, 0, -1}, {0, 1, 0}, {0, 1, -1}},     // T_01
+                                {{0, 0, 0}, {0, 0, -1}, {1, 0, 0}, {1, 0, -1}},     // T_02
+                                {{0, 0, 0}, {0, -1, 0}, {1, 0, 0}, {1, -1, 0}},     // T_12
+                                {{0, 0, 0}, {0, 0, 1}, {0, -1, 0}, {0, -1, 1}},     // T_01^T
+                                {{0, 0, 0}, {0, 0, 1}, {-1, 0, 0}, {-1, 0, 1}},     // T_02^T
+                                {{0, 0, 0}, {0, 1, 0}, {-1, 0, 0}, {-1, 1, 0}}};    // T_12^T
+    return t[b][k][d];
+  }
+  const uchar4* mid;
+  const T* mtab;
+  T s8;   // 1 / 8, with the transforms' scale
+  int cell, lg, msk, x, y, z;
+  __device__ __forceinline__ CrossStencil(const uchar4* ids, const T* tab, int n, int lgn, T s, int c)
+      : mid(ids), mtab(tab), s8(s * (T)0.125), cell(c), lg(lgn), msk(n - 1) {   // n = 2^lgn
+    x = cell & msk;
+    y = (cell >> lg) & msk;
+    z = cell >> (2 * lg);
+  }
+  __device__ __forceinline__ int at(int b, int k) const {   // cell of point k of block b
+    return (((z + ofs(b, k, 0)) & msk) << (2 * lg)) | (((y + ofs(b, k, 1)) & msk) << lg) | ((x + ofs(b, k, 2)) & msk);
+  }
+  // (eps_1)_ij of the material at point set c of cell q; pair 0: 12, 1: 13, 2: 23
+  __device__ __forceinline__ cx<T> off(int q, int c, int pair) const {
+    const uchar4 id = mid[q];
+    const int m = c == 0 ? id.x : (c == 1 ? id.y : id.z);
+    return mk(mtab[9 * m + 3 + 2 * pair], mtab[9 * m + 4 + 2 * pair]);
+  }
+  __device__ __forceinline__ cx<T> own(int b) const { return off(cell, row(b), pair(b)); }
+  // coefficient of point k of block b, at cell q
+  __device__ __forceinline__ cx<T> coef(int b, cx<T> o, int q) const {
+    const cx<T> c = o + off(q, col(b), pair(b));
+    return b < 3 ? scale(c, s8) : mk(c.x * s8, -(c.y * s8));   // (j, i): the conjugate
+  }
+  __device__ __forceinline__ void diagonal(T d[3], T s) const {
+    const uchar4 id = mid[cell];
+    d[0] = mtab[9 * id.x] * s;
+    d[1] = mtab[9 * id.y + 1] * s;
+    d[2] = mtab[9 * id.z + 2] * s;
+  }
+};
+
 // The 24 coefficients of a cell depend on the materials only.  Gathering them
 // (24 ids, 48 table entries) cost four times the 27 field values of a vector,
 // so a thread keeps them in registers and walks the vectors v0, v0 + 1, ... of
-// its group.  Measured at 64^3, 10 complex64 vectors: 61 -> 47 us.
+// its group.  The apply of 10 complex64 vectors of 64^3: 219 -> 210 us.
 template <typename T>
 __global__ void __launch_bounds__(256) crossdof_kernel(const cx<T>* __restrict__ E, cx<T>* __restrict__ Mo,
                                                        const uchar4* __restrict__ mid, const T* __restrict__ mtab, int n,
                                                        int nvec, int group, T s) {
-  const int n3 = n * n * n;
-  const int lg = __ffs(n) - 1;   // n is a power of two
-  const int msk = n - 1;
+  using CS = CrossStencil<T>;
+  const int n3 = n * n * n, lg = __ffs(n) - 1;
   const int v0 = blockIdx.y * group, v1 = v0 + group < nvec ? v0 + group : nvec;
   for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n3; cell += gridDim.x * blockDim.x) {
-    const int x = cell & msk, y = (cell >> lg) & msk, z = cell >> (2 * lg);
-    auto at = [&](int dz, int dy, int dx) -> int {
-      return (((z + dz) & msk) << (2 * lg)) | (((y + dy) & msk) << lg) | ((x + dx) & msk);
-    };
-    // (eps_1)_ij of the material at point set c of cell q; pair 0: 12, 1: 13, 2: 23
-    auto off = [&](int q, int c, int pair) -> cx<T> {
-      const uchar4 id = mid[q];
-      const int m = c == 0 ? id.x : (c == 1 ? id.y : id.z);
-      return mk(mtab[9 * m + 3 + 2 * pair], mtab[9 * m + 4 + 2 * pair]);
-    };
-    // block b: component row_b from component col_b; pair, and the offsets
-    // (dz, dy, dx) of its four points: (i, j) of each pair, then (j, i)
-    constexpr int ROW[6] = {0, 0, 1, 1, 2, 2}, COL[6] = {1, 2, 2, 0, 0, 1}, PAIR[6] = {0, 1, 2, 0, 1, 2};
-    constexpr int OFS[6][4][3] = {{{0, 0, 0}, {0, 0, -1}, {0, 1, 0}, {0, 1, -1}},     // T_01
-                                  {{0, 0, 0}, {0, 0, -1}, {1, 0, 0}, {1, 0, -1}},     // T_02
-                                  {{0, 0, 0}, {0, -1, 0}, {1, 0, 0}, {1, -1, 0}},     // T_12
-                                  {{0, 0, 0}, {0, 0, 1}, {0, -1, 0}, {0, -1, 1}},     // T_01^T
-                                  {{0, 0, 0}, {0, 0, 1}, {-1, 0, 0}, {-1, 0, 1}},     // T_02^T
-                                  {{0, 0, 0}, {0, 1, 0}, {-1, 0, 0}, {-1, 1, 0}}};    // T_12^T
+    const CS cs(mid, mtab, n, lg, s, cell);
     cx<T> cf[6][4];
-    const T s8 = s * (T)0.125;
 #pragma unroll
     for (int b = 0; b < 6; ++b) {
-      const cx<T> own = off(cell, ROW[b], PAIR[b]);
+      const cx<T> own = cs.own(b);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const cx<T> c = own + off(at(OFS[b][k][0], OFS[b][k][1], OFS[b][k][2]), COL[b], PAIR[b]);
-        cf[b][k] = b < 3 ? scale(c, s8) : mk(c.x * s8, -(c.y * s8));   // (j, i): the conjugate
-      }
+      for (int k = 0; k < 4; ++k) cf[b][k] = cs.coef(b, own, cs.at(b, k));
     }
-    const uchar4 id = mid[cell];
-    const T d[3] = {mtab[9 * id.x] * s, mtab[9 * id.y + 1] * s, mtab[9 * id.z + 2] * s};
+    T d[3];
+    cs.diagonal(d, s);
     for (int v = v0; v < v1; ++v) {
       const cx<T>* ev = E + (size_t)v * 3 * n3;
       cx<T> m[3];
@@ -890,12 +919,66 @@ __global__ void __launch_bounds__(256) crossdof_kernel(const cx<T>* __restrict__
       for (int b = 0; b < 6; ++b)
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          m[ROW[b]] = cfma(cf[b][k], ev[(size_t)COL[b] * n3 + at(OFS[b][k][0], OFS[b][k][1], OFS[b][k][2])], m[ROW[b]]);
+          m[CS::row(b)] = cfma(cf[b][k], ev[(size_t)CS::col(b) * n3 + cs.at(b, k)], m[CS::row(b)]);
       cx<T>* mo = Mo + (size_t)v * 3 * n3;
 #pragma unroll
       for (int c = 0; c < 3; ++c) mo[(size_t)c * n3 + cell] = m[c];
     }
   }
+}
+
+// The same for a lone vector, or cells whose vectors go to different CTAs: a
+// coefficient is formed where it is used, with half the registers.
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
+    crossdof_single_kernel(const cx<T>* __restrict__ E, cx<T>* __restrict__ Mo, const uchar4* __restrict__ mid,
+                           const T* __restrict__ mtab, int n, int nvec, T s) {
+  using CS = CrossStencil<T>;
+  const int n3 = n * n * n, lg = __ffs(n) - 1;
+  const size_t total = (size_t)n3 * nvec;
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+    const int cell = (int)(e & (size_t)(n3 - 1)), v = (int)(e >> (3 * lg));
+    const CS cs(mid, mtab, n, lg, s, cell);
+    const cx<T>* ev = E + (size_t)v * 3 * n3;
+    T d[3];
+    cs.diagonal(d, s);
+    cx<T> m[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m[c] = scale(ev[(size_t)c * n3 + cell], d[c]);
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      const cx<T> own = cs.own(b);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int q = cs.at(b, k);
+        m[CS::row(b)] = cfma(cs.coef(b, own, q), ev[(size_t)CS::col(b) * n3 + q], m[CS::row(b)]);
+      }
+    }
+    cx<T>* mo = Mo + (size_t)v * 3 * n3;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) mo[(size_t)c * n3 + cell] = m[c];
+  }
+}
+
+// The stencil pass over nv vectors, in equal groups of up to 16 that share a
+// cell's coefficients.  Small grids take smaller groups: complex64, bound by
+// its loads, needs about four CTAs per SM (152u * 4u); complex128, bound by the
+// FP64 pipe, which forms the coefficients, needs most SMs busy and no more.
+template <typename T>
+cudaError_t launch_crossdof(const cx<T>* E, cx<T>* Mo, const uchar4* mid, const T* mtab, int n, int nv, T s,
+                            cudaStream_t st) {
+  const unsigned cells = ((unsigned)n * n * n + 255) / 256, fill = sizeof(T) == 4 ? 152u * 4u : 152u * 3u / 4u;
+  int group = (nv + (nv + 15) / 16 - 1) / ((nv + 15) / 16);
+  while (group > 1 && cells * (unsigned)((nv + group - 1) / group) < fill) group = (group + 1) / 2;
+  if (group > 1) {
+    group = std::max(group, (nv + 65534) / 65535);   // blockIdx.y is at most 65535
+    crossdof_kernel<T>
+        <<<dim3(cells, (unsigned)((nv + group - 1) / group)), 256, 0, st>>>(E, Mo, mid, mtab, n, nv, group, s);
+  } else {
+    const unsigned blocks = (unsigned)std::min<size_t>((size_t)cells * nv, 152u * 16u);
+    crossdof_single_kernel<T><<<blocks, 256, 0, st>>>(E, Mo, mid, mtab, n, nv, s);
+  }
+  return cudaGetLastError();
 }
 
 // complex128: the pass with its transforms in fixed point (fft_fixed.cuh)
@@ -983,15 +1066,9 @@ cudaError_t run_apply_n(const pcx_ctx* c, const KParams& kp, const void* X, void
       a.in = y;
       if ((e = launch_pass<T, N, 1, OP_INV>(a, tiles, smem, st)) != cudaSuccess) return e;
       if ((e = launch_pass<T, N, 2, OP_PLAIN_INV>(a, tiles, C::SMEM, st)) != cudaSuccess) return e;
-      // groups of up to 16 vectors share a cell's coefficients; small grids
-      // take smaller groups so that every SM has work
-      constexpr unsigned cells = (unsigned)(N * N * N + 255) / 256;
-      int group = nv < 16 ? nv : 16;
-      while (group > 1 && cells * (unsigned)((nv + group - 1) / group) < 152u * 4u) group = (group + 1) / 2;
-      crossdof_kernel<T><<<dim3(cells, (unsigned)((nv + group - 1) / group)), 256, 0, st>>>(
-          y, tmp, static_cast<const uchar4*>(c->dev.mid), static_cast<const T*>(a.mtab), N, nv, group,
-          (T)(1.0 / ((double)N * N * N)));
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = launch_crossdof<T>(y, tmp, static_cast<const uchar4*>(c->dev.mid), static_cast<const T*>(a.mtab), N, nv,
+                                  (T)(1.0 / ((double)N * N * N)), st)) != cudaSuccess)
+        return e;
       a.in = tmp;
       if ((e = launch_pass<T, N, 2, OP_PLAIN_FWD>(a, tiles, C::SMEM, st)) != cudaSuccess) return e;
       a.in = y;

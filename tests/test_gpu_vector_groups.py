@@ -1,0 +1,54 @@
+"""Kernels that take a cell or a mode through a group of vectors (the M_CrossDoF
+stencil, K_P^{-1}): counts that give one vector, full groups and ragged last
+groups, against the oracle for the vectors at the groups' ends and bit for bit
+against the same vectors one at a time.  Tolerances as in test_gpu_apply.py:
+1e-12 (complex128), 2e-5 (complex64) of the largest output."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from oracle import crossdof, fourier, penalty
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = {np.complex64: 2e-5, np.complex128: 1e-12}
+K = np.array([0.6, 1.3, -0.5])
+
+
+@pytest.fixture(scope="module")
+def pcx():
+    from paper_2511_17107_gb300 import pcx as p
+    p.lib()
+    return p
+
+
+def _check(pcx, ctx, call, x, oracle, chunks):
+    dtype = x.dtype.type
+    X = torch.from_numpy(x).cuda()
+    Y = torch.empty_like(X)
+    call(ctx, K, X, Y)
+    one = torch.empty_like(X[:1])
+    for j in range(x.shape[0]):
+        call(ctx, K, X[j:j + 1].contiguous(), one)
+        assert torch.equal(one[0], Y[j]), j
+    for j in sorted({0, x.shape[0] // 2, x.shape[0] - 1}):
+        want = oracle(x[j:j + 1].astype(np.complex128))[0]
+        assert np.abs(Y[j].cpu().numpy() - want).max() <= TOL[dtype] * np.abs(want).max()
+    Z = torch.empty_like(X)
+    for chunk in chunks:
+        pcx.pcx_set_apply_chunk(ctx, chunk)
+        call(ctx, K, X, Z)
+        assert torch.equal(Y, Z), chunk
+    pcx.pcx_set_apply_chunk(ctx, 0)
+
+
+@pytest.mark.parametrize("n,nvec", [(8, 40), (16, 17), (32, 18), (64, 2), (64, 17)])
+@pytest.mark.parametrize("dtype", [np.complex64, np.complex128])
+def test_crossdof(pcx, n, nvec, dtype):
+    s = wl.bcc_gyroid()
+    m = crossdof.CrossDofM(s, n)
+    kap = fourier.kappa(n, s.lattice, K)
+    g = penalty.gamma_practical(K)
+    ctx = pcx.setup_structure(s, n, m_kind=pcx.PCX_M_CROSSDOF)
+    x = wl.random_block(nvec, n, seed=n + nvec).astype(dtype)
+    _check(pcx, ctx, pcx.pcx_apply, x, lambda v: fourier.apply_symbols(v, kap, m.apply, g), (1, 5, nvec))
