@@ -608,18 +608,21 @@ __global__ void __launch_bounds__(Cfg<T, N>::THREADS, 3) pass_kernel(PassArgs a)
 // cost more than the two products of a vector, and the FP64 pipe bounds the
 // complex128 form.  Measured (16 complex128 vectors at 32^3, CTAs of 128 so
 // that the groups of a small grid still reach every SM): 69 -> 40 us. At 128^3,
-// 16 vectors: complex64 406 -> 266 us, complex128 4.32 -> 2.00 ms; one vector 46
-// -> 38 and 279 -> 285 us.
+// 16 vectors: complex64 406 -> 266 us, complex128 4.32 -> 2.00 ms.  A lone
+// vector (in pairs of calls): the entries loaded before kappa is formed, 1 /
+// gamma passed in; complex64 at 128^3 72 -> 41 us, at 256^3 399 -> 150 (172
+// with the loads after kappa); complex128 333 -> 332 us at 128^3.
 template <typename T>
 __global__ void __launch_bounds__(128) precond_kernel(const cx<T>* __restrict__ R, cx<T>* __restrict__ W,
                                                       const cx<T>* __restrict__ lam, int n, int nvec, int group,
-                                                      KParams kp) {
+                                                      KParams kp, T ig) {
   const size_t n3 = (size_t)n * n * n;
   const int lg = __ffs(n) - 1;   // n is a power of two
   const int v0 = blockIdx.y * group, v1 = v0 + group < nvec ? v0 + group : nvec;
-  const T ig = (T)(1.0 / kp.gamma);
   for (size_t mode = (size_t)blockIdx.x * blockDim.x + threadIdx.x; mode < n3; mode += (size_t)gridDim.x * blockDim.x) {
     const int p1 = (int)(mode & (n - 1)), p2 = (int)((mode >> lg) & (n - 1)), p3 = (int)(mode >> (2 * lg));
+    size_t base = (size_t)v0 * 3 * n3 + mode;
+    cx<T> r0 = R[base], r1 = R[base + n3], r2 = R[base + 2 * n3];   // in flight while kappa is formed
     cx<T> kap[3];
     kappa_at<T>(lam, n, kp, p1, p2, p3, kap);
     const T k2 = norm2(kap[0]) + norm2(kap[1]) + norm2(kap[2]);
@@ -627,9 +630,7 @@ __global__ void __launch_bounds__(128) precond_kernel(const cx<T>* __restrict__ 
     const T ik2 = nz ? (T)1 / k2 : (T)0;
     const T cg = ig * penalty_inv_weight(kp, k2) - (T)1;
     const T cs = cg * ik2 * ik2;
-    for (int v = v0; v < v1; ++v) {
-      const size_t base = (size_t)v * 3 * n3 + mode;
-      const cx<T> r0 = R[base], r1 = R[base + n3], r2 = R[base + 2 * n3];
+    for (int v = v0;;) {
       cx<T> w0, w1, w2;
       if (nz) {
         const cx<T> sk = scale(cfma(kap[2], r2, cfma(kap[1], r1, kap[0] * r0)), cs);
@@ -642,6 +643,11 @@ __global__ void __launch_bounds__(128) precond_kernel(const cx<T>* __restrict__ 
       W[base] = w0;
       W[base + n3] = w1;
       W[base + 2 * n3] = w2;
+      if (++v >= v1) break;
+      base += 3 * n3;
+      r0 = R[base];
+      r1 = R[base + n3];
+      r2 = R[base + 2 * n3];
     }
   }
 }
@@ -1237,13 +1243,14 @@ cudaError_t run_precond_t(const pcx_ctx* c, const KParams& kp, const void* R, vo
   // at most 32 CTAs per SM, whose threads go on to further modes: one mode per
   // thread made a single vector of 128^3 76 us instead of 38 (complex64)
   const unsigned cells = (unsigned)std::min<size_t>((n3 + 127) / 128, 152u * 32u);
-  // groups of up to 16 vectors; small grids take smaller ones so that every SM has work
-  int group = nvec < 16 ? nvec : 16;
+  // equal groups of up to 16 vectors; small grids take smaller ones so that every SM has work
+  int group = (nvec + (nvec + 15) / 16 - 1) / ((nvec + 15) / 16);
   while (group > 1 && cells * (unsigned)((nvec + group - 1) / group) < 152u * 4u) group = (group + 1) / 2;
   group = std::max(group, (nvec + 65534) / 65535);   // blockIdx.y is at most 65535
   const void* lam = sizeof(T) == 8 ? c->dev.lam64 : c->dev.lam32;
   fftk::precond_kernel<T><<<dim3(cells, (unsigned)((nvec + group - 1) / group)), 128, 0, s>>>(
-      static_cast<const cx<T>*>(R), static_cast<cx<T>*>(W), static_cast<const cx<T>*>(lam), c->n, nvec, group, kp);
+      static_cast<const cx<T>*>(R), static_cast<cx<T>*>(W), static_cast<const cx<T>*>(lam), c->n, nvec, group, kp,
+      (T)(1.0 / kp.gamma));
   return cudaGetLastError();
 }
 

@@ -52,3 +52,14 @@ def test_crossdof(pcx, n, nvec, dtype):
     ctx = pcx.setup_structure(s, n, m_kind=pcx.PCX_M_CROSSDOF)
     x = wl.random_block(nvec, n, seed=n + nvec).astype(dtype)
     _check(pcx, ctx, pcx.pcx_apply, x, lambda v: fourier.apply_symbols(v, kap, m.apply, g), (1, 5, nvec))
+
+
+@pytest.mark.parametrize("n,nvec", [(8, 1), (16, 33), (32, 5), (64, 1), (64, 17)])
+@pytest.mark.parametrize("dtype", [np.complex64, np.complex128])
+def test_precond(pcx, n, nvec, dtype):
+    s = wl.fcc_air_spheres()
+    kap = fourier.kappa(n, s.lattice, K)
+    g = penalty.gamma_practical(K)
+    ctx = pcx.setup_structure(s, n)
+    x = wl.random_block(nvec, n, seed=n + nvec).astype(dtype)
+    _check(pcx, ctx, pcx.pcx_precond, x, lambda v: fourier.precondition(v, kap, g), ())
