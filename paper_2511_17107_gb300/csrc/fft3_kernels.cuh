@@ -68,11 +68,14 @@ template <> struct YSplit<128> { static constexpr int RA = 16, RB = 8; };
 #ifndef PCX_Z128_MINB
 #define PCX_Z128_MINB 1
 #endif
-template <int N>
+template <int N, bool HALF = false>
 struct ZGeom {
   static constexpr int TN = 2048, E = 16, MINB = 2;
 };
 template <> struct ZGeom<64> { static constexpr int TN = 4096, E = 48, MINB = 2; };
+// Half tiles (same y split, half the columns, ids read in cell order): a lone
+// 64^3 vector has 64 tiles for 152 SMs.  Apply / T0 35.3 / 37.8 -> 31.3 / 32.6 us.
+template <> struct ZGeom<64, true> { static constexpr int TN = 2048, E = 24, MINB = 2; };
 template <> struct ZGeom<128> { static constexpr int TN = PCX_Z128_TN, E = PCX_Z128_E, MINB = PCX_Z128_MINB; };
 
 // Row padding of the z tiles.  Pass B's y DFTs stage two x columns per
@@ -81,9 +84,9 @@ template <> struct ZGeom<128> { static constexpr int TN = PCX_Z128_TN, E = PCX_Z
 // pencil position perm(xo) = xo / 2 + H (xo % 2), so the two columns of a
 // pair land H apart, and with a row stride SN = H (mod 16) the half-warp's
 // 8-byte words n SN + xp (+ H) fall in 16 distinct bank pairs.
-template <int N>
+template <int N, bool HALF = false>
 struct ZPad {
-  static constexpr int TPZ = ZGeom<N>::TN / N;
+  static constexpr int TPZ = ZGeom<N, HALF>::TN / N;
   static constexpr int H = TPZ / YSplit<N>::RB / 2;
   static constexpr int R = ((H - TPZ) % 16 + 16) % 16;
   static constexpr int V = R == 0 ? 16 : R;
@@ -97,10 +100,10 @@ __host__ __device__ constexpr int zcol_of(int q) {     // tile column at pencil 
   return q < TPX / 2 ? 2 * q : 2 * (q - TPX / 2) + 1;
 }
 
-template <typename T, int N>
+template <typename T, int N, bool HALF = false>
 struct Cfg3 {
   using C = Cfg<T, N>;                                           // x tiles (passes A and C)
-  using CZ = CfgG<T, N, ZGeom<N>::TN, ZGeom<N>::E, ZPad<N>::V>;  // z tiles (pass B)
+  using CZ = CfgG<T, N, ZGeom<N, HALF>::TN, ZGeom<N, HALF>::E, ZPad<N, HALF>::V>;  // z tiles (pass B)
   static constexpr int TP = C::TP;                  // pencils (rows) per x tile
   static constexpr int THREADS = C::THREADS;
   static constexpr int TPZ = CZ::TP;                // pencils per z tile
@@ -124,9 +127,10 @@ template <int OP>
 __host__ __device__ constexpr bool is_z_op() {
   return OP == OP_SANDWICH || OP == OP_SANDWICH_EPS;
 }
-template <typename T, int N, int OP>
+// z passes: XV = 1 runs half tiles
+template <typename T, int N, int OP, int XV>
 __host__ __device__ constexpr int pass3_threads() {
-  return is_z_op<OP>() ? Cfg3<T, N>::THREADSZ : Cfg3<T, N>::THREADS;
+  return is_z_op<OP>() ? Cfg3<T, N, XV == 1>::THREADSZ : Cfg3<T, N>::THREADS;
 }
 // Kernel variants the autotuner chooses between at run time (the tile
 // shapes themselves are fixed by the geometry above, which the pass-B id
@@ -145,7 +149,7 @@ template <> struct XVar<2> { static constexpr int PF = 6, MINB = 2; };
 // are in pcx_internal.h, for the host side)
 template <typename T, int N, int OP, int XV>
 __host__ __device__ constexpr int pass3_minb() {
-  return is_z_op<OP>() ? ZGeom<N>::MINB : XVar<XV>::MINB;
+  return is_z_op<OP>() ? ZGeom<N, XV == 1>::MINB : XVar<XV>::MINB;
 }
 
 // Row of pencil t of x tile `tile` (within one vector): z, y, and the n2
@@ -444,9 +448,9 @@ __device__ __forceinline__ V ld_tab(const V* p) {
 // kernel and the warp-specialised persistent one.  tile = k1 (N / TPX) + xr;
 // pencil t = k2 TPX + q holds tile column xo = zcol_of(q) of real row
 // y = k1 + RA k2, at x = xr TPX + xo.
-template <typename T, int N, int OP>
+template <typename T, int N, int OP, bool HALF = false>
 struct ZTile {
-  using C3 = Cfg3<T, N>;
+  using C3 = Cfg3<T, N, HALF>;
   using C = typename C3::CZ;
   using TL = Tile<T, N, 2, C>;
   static constexpr int TP = C::TP, RA = C3::RA, RB = C3::RB, TPX = C3::TPX;
@@ -549,7 +553,8 @@ struct ZTile {
         T d1, d2, d3;
         cx<T> o12, o13, o23;
         if (tid3) {
-          const uchar4 id = tid3[n * TP + t];
+          // tid3: the ids in tile order; for half tiles in cell order
+          const uchar4 id = tid3[HALF ? n * N2 + (k1 + RA * (t / TPX)) * N + x0 + zcol_of<TPX>(t % TPX) : n * TP + t];
           d1 = ld_tab<GTAB>(mtab + 12 * id.x);
           d2 = ld_tab<GTAB>(mtab + 12 * id.y + 1);
           d3 = ld_tab<GTAB>(mtab + 12 * id.z + 2);
@@ -647,9 +652,9 @@ struct ZTile {
 };
 
 template <typename T, int N, int OP, int XV>
-__global__ void __launch_bounds__(pass3_threads<T, N, OP>(), pass3_minb<T, N, OP, XV>()) pass3_kernel(PassArgs a) {
-  constexpr bool ZP = is_z_op<OP>();
-  using C3 = Cfg3<T, N>;
+__global__ void __launch_bounds__(pass3_threads<T, N, OP, XV>(), pass3_minb<T, N, OP, XV>()) pass3_kernel(PassArgs a) {
+  constexpr bool ZP = is_z_op<OP>(), HALF = ZP && XV == 1;
+  using C3 = Cfg3<T, N, HALF>;
   using C = std::conditional_t<ZP, typename C3::CZ, typename C3::C>;
   constexpr int AXIS = ZP ? 2 : 0;
   using TL = Tile<T, N, AXIS, C>;
@@ -693,7 +698,7 @@ __global__ void __launch_bounds__(pass3_threads<T, N, OP>(), pass3_minb<T, N, OP
     }
   } else {
     // ================= z tiles: pass B =================
-    using ZT = ZTile<T, N, OP>;
+    using ZT = ZTile<T, N, OP, HALF>;
     constexpr int TPX = C3::TPX;
     const int k1 = tile / (N / TPX), x0 = (tile % (N / TPX)) * TPX;
     if (a.mid && !ZT::GTAB) ZT::stage_mtab(mtab, a.mtab, a.n_mat, threadIdx.x, C::THREADS);
@@ -701,9 +706,9 @@ __global__ void __launch_bounds__(pass3_threads<T, N, OP>(), pass3_minb<T, N, OP
     const cx<T>* twz = ZT::GTW ? gtw : tw;
     ZT::template load<C::THREADS>(s, in, k1, x0, threadIdx.x);
     __syncthreads();   // the tile, the twiddles and the material table
-    const uchar4* mid3 = static_cast<const uchar4*>(a.mid3);
-    ZT::template transform<CtaSync>(s, twz, mt, mid3 ? mid3 + (size_t)tile * TP * N : nullptr,
-                                    static_cast<const T*>(a.M), k1, x0);
+    const uchar4* ids = static_cast<const uchar4*>(HALF ? a.mid : a.mid3);
+    if (!HALF && ids) ids += (size_t)tile * TP * N;
+    ZT::template transform<CtaSync>(s, twz, mt, ids, static_cast<const T*>(a.M), k1, x0);
     ZT::template store<C::THREADS>(s, twz, out, k1, x0, threadIdx.x);
   }
 }
@@ -886,8 +891,8 @@ size_t mtab_smem(int n_mat) {
 // table).
 template <typename T, int N, int OP, int XV>
 cudaError_t launch_pass3_tile(const PassArgs& a, int nv, cudaStream_t st) {
-  using C3 = Cfg3<T, N>;
   constexpr bool ZP = is_z_op<OP>();
+  using C3 = Cfg3<T, N, ZP && XV == 1>;
   size_t smem;
   if constexpr (ZP)
     smem = C3::ZSMEM_TILE + (size_t)N * sizeof(cx<T>) + mtab_smem<T, N, OP>(a.n_mat);
@@ -897,7 +902,7 @@ cudaError_t launch_pass3_tile(const PassArgs& a, int nv, cudaStream_t st) {
   auto kern = pass3_kernel<T, N, OP, XV>;
   cudaError_t e = raise_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)tiles, pass3_threads<T, N, OP>(), smem, st>>>(a);
+  kern<<<(unsigned)tiles, pass3_threads<T, N, OP, XV>(), smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -960,6 +965,14 @@ cudaError_t launch_pass3(const PassArgs& a, int nv, cudaStream_t st, int xv, int
     // 128-point tiles, of which one fills it, take the other kernel
     if constexpr (2 * Cfg3<T, N>::ZSMEM_TILE + N * sizeof(cx<T>) <= (size_t)227 * 1024) {
       if (zv == 1) return launch_pass3_ws<T, N, OP>(a, nv, st);
+    }
+    if constexpr (N == 64) {
+      // half tiles where each of them still gets an SM of its own (one vector)
+      int dev = 0, sms = 0;
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      if ((long long)nv * Cfg3<T, N, true>::ZTILES <= sms) return launch_pass3_tile<T, N, OP, 1>(a, nv, st);
     }
     return launch_pass3_tile<T, N, OP, 0>(a, nv, st);
   } else {

@@ -63,3 +63,22 @@ def test_precond(pcx, n, nvec, dtype):
     ctx = pcx.setup_structure(s, n)
     x = wl.random_block(nvec, n, seed=n + nvec).astype(dtype)
     _check(pcx, ctx, pcx.pcx_precond, x, lambda v: fourier.precondition(v, kap, g), ())
+
+
+@pytest.mark.parametrize("call", ["pcx_apply", "pcx_sandwich_precond"])
+@pytest.mark.parametrize("dense", [False, True])
+def test_lone_vector_of_the_three_pass_chain(pcx, call, dense):
+    """A lone 64^3 complex64 vector runs half tiles in the z pass: same bits as in a block."""
+    n = 64
+    s = wl.fcc_air_spheres()
+    ctx = pcx.setup_structure(s, n)
+    if dense:
+        ctx = pcx.pcx_setup(n, lattice=s.lattice, cell_blocks=pcx.pcx_cell_blocks(ctx)[0])
+    x = wl.random_block(3, n, seed=3).astype(np.complex64)
+    X = torch.from_numpy(x).cuda()
+    Y = torch.empty_like(X)
+    getattr(pcx, call)(ctx, K, X, Y)
+    one = torch.empty_like(X[:1])
+    for j in range(3):
+        getattr(pcx, call)(ctx, K, X[j:j + 1].contiguous(), one)
+        assert torch.equal(one[0], Y[j]), j
