@@ -214,7 +214,9 @@ pcx_status pcx_symbols(const pcx_ctx* ctx, const double k[3], double gamma,
 pcx_status pcx_set_apply_chunk(pcx_ctx* ctx, int chunk);
 
 /* The chunk pcx_apply uses for `precision`: a block of nvec vectors runs as
- * ceil(nvec / chunk) sweeps of the passes, of equal size.  0 if ctx is NULL. */
+ * ceil(nvec / chunk) sweeps of the passes, of equal size (with the default
+ * chunk, complex64 blocks of 128^3 that would not fill more waves in one sweep
+ * run one vector at a time).  0 if ctx is NULL. */
 int pcx_get_apply_chunk(const pcx_ctx* ctx, int precision);
 
 /*

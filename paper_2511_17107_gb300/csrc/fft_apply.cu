@@ -71,6 +71,21 @@ int apply_chunk(const pcx_ctx* c, int precision) {
   return (int)(fit < 1 ? 1 : (fit > 4096 ? 4096 : fit));
 }
 
+// Vectors per launch for a block of nvec.  One launch for the whole block pays
+// by the waves it saves.  Two or three 128^3 vectors save none in pass B (256
+// tiles a vector, one per SM), and one vector at a time finds its intermediates
+// in L2: complex64, 2 and 3 vectors 236 and 345 us in one launch, 225 and 334
+// one by one (four: 428 and 445).
+static int launch_chunk(const pcx_ctx* c, int precision, int nvec) {
+  const int chunk = apply_chunk(c, precision);
+  if (c->apply_chunk > 0 || nvec > chunk || c->sms < 1 || c->n != 128 ||
+      effective_apply_path(c, precision) != PCX_APPLY_THREE_PASS)
+    return chunk;
+  const long long tiles = (long long)c->n * c->n / 64;
+  const long long waves = (nvec * tiles + c->sms - 1) / c->sms, single = (tiles + c->sms - 1) / c->sms;
+  return waves < nvec * single ? chunk : 1;
+}
+
 cudaError_t raise_dyn_smem(const void* func, size_t bytes) {
   struct Entry {
     const void* f;
@@ -115,7 +130,7 @@ size_t apply_scratch_bytes(const pcx_ctx* c, int precision, int nvec) {
 cudaError_t launch_apply_scratch(const pcx_ctx* c, const KParams& kp, const void* X, void* Y, int nvec, int precision,
                                  void* scratch, cudaStream_t s) {
   if (nvec == 0) return cudaSuccess;
-  const int chunk = apply_chunk(c, precision);
+  const int chunk = launch_chunk(c, precision, nvec);
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kp, X, Y, nvec, chunk, scratch, s)
                                : dispatch_apply<float>(c, kp, X, Y, nvec, chunk, scratch, s);
 }
@@ -149,7 +164,7 @@ cudaError_t launch_apply_noalloc(const pcx_ctx* c, const KParams& kp, const void
   void* scratch = nullptr;
   cudaError_t e = noalloc_scratch(&scratch);
   if (e != cudaSuccess) return e;
-  int chunk = apply_chunk(c, precision);
+  int chunk = launch_chunk(c, precision, nvec);
   const int fit = (int)((size_t)PCX_NOALLOC_SCRATCH_BYTES / per_vec);
   if (chunk > fit) chunk = fit;
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kp, X, Y, nvec, chunk, scratch, s)
@@ -221,7 +236,7 @@ cudaError_t launch_t0(pcx_ctx* c, const KParams& kp, const void* R, void* W, int
   if (nvec == 0) return cudaSuccess;
   cudaError_t e = ensure_scratch(c, precision, nvec);
   if (e != cudaSuccess) return e;
-  const int chunk = apply_chunk(c, precision);
+  const int chunk = launch_chunk(c, precision, nvec);
   return precision == PCX_FP64
              ? run_apply_t<double>(c, kp, R, W, nvec, chunk, c->scratch, nullptr, 1, s, true)
              : run_apply_t<float>(c, kp, R, W, nvec, chunk, c->scratch, nullptr, 1, s, true);
@@ -230,7 +245,7 @@ cudaError_t launch_t0(pcx_ctx* c, const KParams& kp, const void* R, void* W, int
 cudaError_t launch_t0_scratch(const pcx_ctx* c, const KParams& kp, const void* R, void* W, int nvec, int precision,
                               void* scratch, cudaStream_t s) {
   if (nvec == 0) return cudaSuccess;
-  const int chunk = apply_chunk(c, precision);
+  const int chunk = launch_chunk(c, precision, nvec);
   return precision == PCX_FP64 ? run_apply_t<double>(c, kp, R, W, nvec, chunk, scratch, nullptr, 1, s, true)
                                : run_apply_t<float>(c, kp, R, W, nvec, chunk, scratch, nullptr, 1, s, true);
 }
@@ -304,7 +319,7 @@ cudaError_t launch_apply_kbatch(pcx_ctx* c, const KParams* kps_host, int nk, int
   // pageable source: the call returns once the table is staged
   if ((e = cudaMemcpyAsync(c->ktab, kps_host, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   if ((e = ensure_scratch(c, precision, nvec)) != cudaSuccess) return e;
-  const int chunk = apply_chunk(c, precision);
+  const int chunk = launch_chunk(c, precision, nvec);
   const KParams* kt = static_cast<const KParams*>(c->ktab);
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kps_host[0], X, Y, nvec, chunk, c->scratch, s, kt, vec_per_k)
                                : dispatch_apply<float>(c, kps_host[0], X, Y, nvec, chunk, c->scratch, s, kt, vec_per_k);

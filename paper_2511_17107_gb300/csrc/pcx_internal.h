@@ -82,6 +82,7 @@ struct pcx_ctx {
   void* scratch = nullptr;     // gamma kappa.x carried from pass 1 to pass 5
   size_t scratch_bytes = 0;
   size_t l2_bytes = 0;
+  int sms = 0;
   // k table of the k-batched apply (device, grown on demand)
   void* ktab = nullptr;
   size_t ktab_bytes = 0;

@@ -552,6 +552,7 @@ pcx_status setup_context(const pcx_setup_desc* d, pcx_ctx* c) {
   {
     int l2 = 0;
     if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device) == cudaSuccess) c->l2_bytes = (size_t)l2;
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   }
   return PCX_OK;
 cuda_error:

@@ -82,3 +82,18 @@ def test_lone_vector_of_the_three_pass_chain(pcx, call, dense):
     for j in range(3):
         getattr(pcx, call)(ctx, K, X[j:j + 1].contiguous(), one)
         assert torch.equal(one[0], Y[j]), j
+
+
+@pytest.mark.parametrize("nvec", [2, 3, 4])
+def test_few_vectors_at_128(pcx, nvec):
+    """Two and three 128^3 vectors go one by one, four in one launch: same bits either way."""
+    n = 128
+    ctx = pcx.setup_structure(wl.diamond_rods(), n)
+    X = torch.from_numpy(wl.random_block(nvec, n, seed=nvec).astype(np.complex64)).cuda()
+    for call in (pcx.pcx_apply, pcx.pcx_sandwich_precond):
+        out = []
+        for chunk in (0, 1, nvec):
+            pcx.pcx_set_apply_chunk(ctx, chunk)
+            out.append(torch.empty_like(X))
+            call(ctx, K, X, out[-1])
+        assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
