@@ -308,6 +308,9 @@ pcx_status pcx_set_apply_graphs(pcx_ctx* ctx, int enable);
  *                         the intermediates kept in place in Y; complex64 at
  *                         N = 32, 64, 128 (elsewhere the five-pass chain runs);
  *   PCX_APPLY_AUTO        (default) the three-pass form where it exists.
+ * complex64 vectors of 8^3 and 16^3 run the arithmetic of the five passes in
+ * one launch, a block per vector, whatever the path and the chunk, and use no
+ * scratch (pcx_get_apply_path reports the five-pass form there).
  * Both compute the same operator (Sec. 2.4 eq. matrixfree_kcform); the
  * rounding differs.  M_CrossDoF contexts always use their seven-pass chain.
  * PCX_EINVAL for another value.

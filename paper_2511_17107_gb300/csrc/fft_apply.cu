@@ -71,12 +71,17 @@ int apply_chunk(const pcx_ctx* c, int precision) {
   return (int)(fit < 1 ? 1 : (fit > 4096 ? 4096 : fit));
 }
 
+// complex64 vectors of 8^3 and 16^3 run the one-launch kernel (fft_small.cuh;
+// not the M_CrossDoF apply): no scratch, any number of vectors per launch.
+bool one_launch(const pcx_ctx* c, int precision) { return precision == PCX_FP32 && c->n <= 16; }
+
 // Vectors per launch for a block of nvec.  One launch for the whole block pays
 // by the waves it saves.  Two or three 128^3 vectors save none in pass B (256
 // tiles a vector, one per SM), and one vector at a time finds its intermediates
 // in L2: complex64, 2 and 3 vectors 236 and 345 us in one launch, 225 and 334
 // one by one (four: 428 and 445).
-static int launch_chunk(const pcx_ctx* c, int precision, int nvec) {
+static int launch_chunk(const pcx_ctx* c, int precision, int nvec, bool t0) {
+  if (one_launch(c, precision) && (t0 || c->m_kind != PCX_M_CROSSDOF)) return nvec;
   const int chunk = apply_chunk(c, precision);
   if (c->apply_chunk > 0 || nvec > chunk || c->sms < 1 || c->n != 128 ||
       effective_apply_path(c, precision) != PCX_APPLY_THREE_PASS)
@@ -121,6 +126,7 @@ int effective_apply_path(const pcx_ctx* c, int precision) {
 // gamma kappa.x per vector of a chunk, and for M_CrossDoF the real-space
 // field of the stencil pass (3 N^3) after it
 size_t apply_scratch_bytes(const pcx_ctx* c, int precision, int nvec) {
+  if (one_launch(c, precision) && c->m_kind != PCX_M_CROSSDOF) return 0;
   const int chunk = apply_chunk(c, precision);
   const int nv = nvec < chunk ? nvec : chunk;
   const size_t per = (size_t)c->n * c->n * c->n * (precision == PCX_FP64 ? 16 : 8);
@@ -130,7 +136,7 @@ size_t apply_scratch_bytes(const pcx_ctx* c, int precision, int nvec) {
 cudaError_t launch_apply_scratch(const pcx_ctx* c, const KParams& kp, const void* X, void* Y, int nvec, int precision,
                                  void* scratch, cudaStream_t s) {
   if (nvec == 0) return cudaSuccess;
-  const int chunk = launch_chunk(c, precision, nvec);
+  const int chunk = launch_chunk(c, precision, nvec, false);
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kp, X, Y, nvec, chunk, scratch, s)
                                : dispatch_apply<float>(c, kp, X, Y, nvec, chunk, scratch, s);
 }
@@ -164,9 +170,9 @@ cudaError_t launch_apply_noalloc(const pcx_ctx* c, const KParams& kp, const void
   void* scratch = nullptr;
   cudaError_t e = noalloc_scratch(&scratch);
   if (e != cudaSuccess) return e;
-  int chunk = launch_chunk(c, precision, nvec);
+  int chunk = launch_chunk(c, precision, nvec, false);
   const int fit = (int)((size_t)PCX_NOALLOC_SCRATCH_BYTES / per_vec);
-  if (chunk > fit) chunk = fit;
+  if (chunk > fit && !(one_launch(c, precision) && c->m_kind != PCX_M_CROSSDOF)) chunk = fit;
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kp, X, Y, nvec, chunk, scratch, s)
                                : dispatch_apply<float>(c, kp, X, Y, nvec, chunk, scratch, s);
 }
@@ -184,7 +190,7 @@ cudaError_t ensure_scratch(pcx_ctx* c, int precision, int nvec) {
     c->scratch = nullptr;
     c->scratch_bytes = 0;
     e = cudaMalloc(&c->scratch, need);
-    if (e == cudaErrorMemoryAllocation && !c->small_scratch) {   // smaller chunks from now on
+    if (e == cudaErrorMemoryAllocation && !c->small_scratch && c->apply_chunk <= 0) {   // smaller chunks from now on
       cudaGetLastError();
       c->small_scratch = 1;
       need = apply_scratch_bytes(c, precision, nvec);
@@ -236,7 +242,7 @@ cudaError_t launch_t0(pcx_ctx* c, const KParams& kp, const void* R, void* W, int
   if (nvec == 0) return cudaSuccess;
   cudaError_t e = ensure_scratch(c, precision, nvec);
   if (e != cudaSuccess) return e;
-  const int chunk = launch_chunk(c, precision, nvec);
+  const int chunk = launch_chunk(c, precision, nvec, true);
   return precision == PCX_FP64
              ? run_apply_t<double>(c, kp, R, W, nvec, chunk, c->scratch, nullptr, 1, s, true)
              : run_apply_t<float>(c, kp, R, W, nvec, chunk, c->scratch, nullptr, 1, s, true);
@@ -245,7 +251,7 @@ cudaError_t launch_t0(pcx_ctx* c, const KParams& kp, const void* R, void* W, int
 cudaError_t launch_t0_scratch(const pcx_ctx* c, const KParams& kp, const void* R, void* W, int nvec, int precision,
                               void* scratch, cudaStream_t s) {
   if (nvec == 0) return cudaSuccess;
-  const int chunk = launch_chunk(c, precision, nvec);
+  const int chunk = launch_chunk(c, precision, nvec, true);
   return precision == PCX_FP64 ? run_apply_t<double>(c, kp, R, W, nvec, chunk, scratch, nullptr, 1, s, true)
                                : run_apply_t<float>(c, kp, R, W, nvec, chunk, scratch, nullptr, 1, s, true);
 }
@@ -319,7 +325,7 @@ cudaError_t launch_apply_kbatch(pcx_ctx* c, const KParams* kps_host, int nk, int
   // pageable source: the call returns once the table is staged
   if ((e = cudaMemcpyAsync(c->ktab, kps_host, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   if ((e = ensure_scratch(c, precision, nvec)) != cudaSuccess) return e;
-  const int chunk = launch_chunk(c, precision, nvec);
+  const int chunk = launch_chunk(c, precision, nvec, false);
   const KParams* kt = static_cast<const KParams*>(c->ktab);
   return precision == PCX_FP64 ? dispatch_apply<double>(c, kps_host[0], X, Y, nvec, chunk, c->scratch, s, kt, vec_per_k)
                                : dispatch_apply<float>(c, kps_host[0], X, Y, nvec, chunk, c->scratch, s, kt, vec_per_k);

@@ -133,6 +133,7 @@ cudaError_t launch_apply_scratch(const pcx_ctx* c, const KParams& kp, const void
 cudaError_t launch_apply_noalloc(const pcx_ctx* c, const KParams& kp, const void* X, void* Y, int nvec,
                                  int precision, cudaStream_t s);
 int apply_chunk(const pcx_ctx* c, int precision);
+bool one_launch(const pcx_ctx* c, int precision);   // complex64 at N = 8, 16 (not the M_CrossDoF apply)
 // pass structure the apply runs: PCX_APPLY_FIVE_PASS, PCX_APPLY_THREE_PASS, or 7 (M_CrossDoF)
 int effective_apply_path(const pcx_ctx* c, int precision);
 // dev.mid3 from dev.mid (allocates; a no-op where the three-pass form does not exist)

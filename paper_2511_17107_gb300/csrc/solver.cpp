@@ -903,7 +903,7 @@ pcx_status solve_concurrent(KSolve& base, const double* kpts, int nk, double pen
     const size_t scr = std::max(apply_scratch_bytes(c, PCX_FP64, n3cols), apply_scratch_bytes(c, PCX_FP32, n3cols));
     e = cudaSuccess;
     for (int w = 0; w < conc && e == cudaSuccess; ++w) e = ascrs[w].alloc(scr);
-    if (e != cudaErrorMemoryAllocation || c->small_scratch) break;
+    if (e != cudaErrorMemoryAllocation || c->small_scratch || c->apply_chunk > 0) break;
     cudaGetLastError();
     c->small_scratch = 1;
     ascrs = std::vector<DevBuf>(conc);
