@@ -406,9 +406,10 @@ typedef struct {
  * blocks of nvec vectors at `precision`: for each pass structure the
  * context has (the five-pass chain, and the three-pass one where it
  * exists; see pcx_set_apply_path), every chunk size 1, 2, 4, ... <=
- * min(nvec, 64) (and nvec) is timed with CUDA events on `stream` (two warm
+ * min(nvec, 64) (and nvec), and what an untuned context would use, is timed with CUDA events on `stream` (two warm
  * and three timed applies on random vectors); when the three-pass chain
- * wins, every pair of its kernel variants (pcx_set_apply_variant) at the
+ * wins, every pair of its kernel variants (pcx_set_apply_variant; none that runs
+ * as another) at the
  * best chunk; then graph replay of the best configuration when `stream` is
  * not the default stream.  The choice is applied to the context (as
  * pcx_set_apply_path / pcx_set_apply_chunk / pcx_set_apply_variant /

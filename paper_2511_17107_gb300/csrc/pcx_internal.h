@@ -136,6 +136,8 @@ int apply_chunk(const pcx_ctx* c, int precision);
 bool one_launch(const pcx_ctx* c, int precision);   // complex64 at N = 8, 16 (not the M_CrossDoF apply)
 // pass structure the apply runs: PCX_APPLY_FIVE_PASS, PCX_APPLY_THREE_PASS, or 7 (M_CrossDoF)
 int effective_apply_path(const pcx_ctx* c, int precision);
+// pass B's kernel that runs: variant 1 needs two tiles in an SM's shared memory, which those of N = 128 are too large for
+inline int effective_z_variant(const pcx_ctx* c) { return c->n == 128 ? 0 : (c->z3_variant >= 0 ? c->z3_variant : PCX_Z3_VARIANT); }
 // dev.mid3 from dev.mid (allocates; a no-op where the three-pass form does not exist)
 cudaError_t build_pass3_ids(pcx_ctx* c);
 // k-batched apply: nk groups of vec_per_k vectors, group i at kps_host[i]

@@ -112,6 +112,7 @@ cudaError_t autotune_apply(pcx_ctx* c, int precision, int nvec, cudaStream_t s, 
     c->apply_path = r.path;
     c->x3_variant = r.x_variant;
     c->z3_variant = r.z_variant;
+    if (r.z_variant >= 0) c->z3_variant = r.z_variant = effective_z_variant(c);   // lines of earlier builds
     if (out) *out = r;
     return cudaSuccess;
   }
@@ -149,8 +150,21 @@ cudaError_t autotune_apply(pcx_ctx* c, int precision, int nvec, cudaStream_t s, 
     *ms = f / reps;
     return cudaSuccess;
   };
-  for (int ch = 1; ch <= 64 && ch <= nvec; ch *= 2) cands.push_back(ch);
-  if (std::find(cands.begin(), cands.end(), nvec) == cands.end() && nvec <= 64) cands.push_back(nvec);
+  // chunks: powers of two, the whole block where it is small, and what an
+  // untuned context would use
+  {
+    const int keep = c->apply_chunk;
+    c->apply_chunk = 0;
+    const int untuned = std::min(apply_chunk(c, precision), nvec);
+    c->apply_chunk = keep;
+    if (!one_launch(c, precision) || c->m_kind == PCX_M_CROSSDOF) {
+      for (int ch = 1; ch <= 64 && ch <= nvec; ch *= 2) cands.push_back(ch);
+      if (nvec <= 64) cands.push_back(nvec);
+    }
+    cands.push_back(untuned);
+    std::sort(cands.begin(), cands.end());
+    cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
+  }
   CKT(cudaMalloc(&X, vbytes * nvec));
   CKT(cudaMalloc(&Y, vbytes * nvec));
   CKT(launch_fill_random(X, nvec, vbytes / (precision == PCX_FP64 ? 16 : 8), 12345, precision, s));
@@ -187,6 +201,7 @@ cudaError_t autotune_apply(pcx_ctx* c, int precision, int nvec, cudaStream_t s, 
         if (xv == PCX_X3_VARIANT && zv == PCX_Z3_VARIANT) continue;
         c->x3_variant = xv;
         c->z3_variant = zv;
+        if (effective_z_variant(c) != zv) continue;   // runs as another one
         double ms = 0;
         CKT(time_apply(&ms));
         ++r.candidates;

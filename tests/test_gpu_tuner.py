@@ -16,6 +16,22 @@ def pcx():
     return p
 
 
+def test_the_untuned_chunk_is_among_the_candidates(pcx):
+    """Chunks 1, 2, ..., 64 and the 200 of an untuned context, for both pass structures."""
+    ctx = pcx.setup_structure(wl.sc_gyro_sphere(), 32)
+    assert pcx.pcx_get_apply_chunk(ctx, pcx.PCX_FP32) >= 200
+    r = pcx.pcx_autotune(ctx, pcx.PCX_FP32, 200)
+    assert r["candidates"] == 2 * 8 + (7 if r["path"] == pcx.PCX_APPLY_THREE_PASS else 0)
+
+
+def test_a_variant_that_runs_as_another_is_not_timed(pcx):
+    """At N = 128 pass B has one kernel: four x variants, z variant 0 reported."""
+    ctx = pcx.setup_structure(wl.diamond_rods(), 128)
+    r = pcx.pcx_autotune(ctx, pcx.PCX_FP32, 2)
+    three = r["path"] == pcx.PCX_APPLY_THREE_PASS
+    assert r["candidates"] == 2 * 2 + (3 if three else 0) and r["z_variant"] == (0 if three else -1)
+
+
 @pytest.mark.parametrize("n", [8, 16])
 def test_one_launch_applies(pcx, n):
     """Nothing to choose, no scratch, and a set chunk does not split the block: same bits."""
@@ -29,6 +45,7 @@ def test_one_launch_applies(pcx, n):
     pcx.pcx_apply(ctx, K, X, Y)
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] == free
+    assert pcx.pcx_autotune(ctx, pcx.PCX_FP32, 256)["candidates"] == 1
     pcx.pcx_set_apply_chunk(ctx, 7)
     pcx.pcx_apply(ctx, K, X, Z)
     assert torch.equal(Y, Z)
