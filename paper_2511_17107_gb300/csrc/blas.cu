@@ -372,62 +372,72 @@ __global__ void __launch_bounds__(256) combine_add32_kernel(const cx<float>* __r
   }
 }
 
-// A few FP32 squares as a double-float pair.  A square that takes the pair
-// beyond the FP32 range (or is Inf or NaN itself) goes to the FP64 sum alone,
-// so the sum has the range of FP64 and infinities stay infinite.
-struct SquareSum {
-  dfloat::DF p{0.f, 0.f};
-  __device__ __forceinline__ void add(float q, double& total) {
-    if (!(__fadd_rn(p.s, q) <= 3.402823466e38f)) {
-      total += (double)q;
-      return;
-    }
-    dfloat::add(p, q, 0.f);
-  }
-  __device__ __forceinline__ void flush(double& total) {
+// total += eight FP32 squares: gathered in a double-float pair on the FP32 pipes
+// (the pair rounds at 2^-48, each square at 2^-24) and added once.  Squares that
+// take the pair beyond the FP32 range, or are Inf or NaN themselves, are added one
+// by one, so the sum has the range of FP64 and infinities stay infinite.
+__device__ __forceinline__ void add_squares(double& total, const float q[8]) {
+  dfloat::DF p{q[0], 0.f};
+#pragma unroll
+  for (int u = 1; u < 8; ++u) dfloat::add(p, q[u], 0.f);
+  if (p.s <= 3.402823466e38f) {
     total += (double)p.s + (double)p.c;
-    p = dfloat::DF{0.f, 0.f};
+  } else {
+    for (int u = 0; u < 8; ++u) total += (double)q[u];
   }
-};
+}
 
 // ---------------------------------------------------------------------------
 // Residual R_j = AX_j - theta_j X_j with ||R_j||^2 and ||X_j||^2 (FP64).
+// BATCH (complex64): eight entries of a thread at a time.
 // ---------------------------------------------------------------------------
-template <typename T>
+template <typename T, bool BATCH>
 __global__ void __launch_bounds__(256) residual_kernel(const cx<T>* __restrict__ X, const cx<T>* AX, const double* theta,
                                                        cx<T>* R, double* norms, int nvec, size_t L) {
   const int j = blockIdx.y;
   const T th = (T)theta[j];
   // squares summed per thread in FP64.  complex64: two FP64 conversions and
   // additions per entry bound the kernel at 0.80 ms for 16 columns of 3 128^3;
-  // so eight squares gather in a double-float pair on the FP32 pipes before
-  // they are added (the pair rounds at 2^-48, each FP32 square at 2^-24).
+  // eight entries at a time it takes 0.37 (columns of at least as many a thread).
   double rr = 0.0, xx = 0.0;
-  SquareSum rf, xf;
-  int pending = 0;
   const cx<T>* x = X + (size_t)j * L;
   const cx<T>* ax = AX + (size_t)j * L;
   cx<T>* r = R + (size_t)j * L;
-  for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < L; l += (size_t)gridDim.x * blockDim.x) {
-    const cx<T> xv = x[l], av = ax[l];
-    const cx<T> rv = mk(fma(-th, xv.x, av.x), fma(-th, xv.y, av.y));
-    r[l] = rv;
-    if constexpr (sizeof(T) == 4) {
-      rf.add(norm2(rv), rr);
-      xf.add(norm2(xv), xx);
-      if (++pending == 8) {
-        rf.flush(rr);
-        xf.flush(xx);
-        pending = 0;
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  if constexpr (BATCH) {
+    for (size_t l0 = first; l0 < L; l0 += 8 * stride) {
+      cx<T> xv[8], av[8];   // R may be AX: all eight are read before any is written
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const size_t l = l0 + u * stride;
+        xv[u] = l < L ? x[l] : mk((T)0, (T)0);
+        av[u] = l < L ? ax[l] : mk((T)0, (T)0);
       }
-    } else {
-      rr = fma(rv.x, rv.x, fma(rv.y, rv.y, rr));
-      xx = fma(xv.x, xv.x, fma(xv.y, xv.y, xx));
+      float qr[8], qx[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const size_t l = l0 + u * stride;
+        const cx<T> rv = mk(fma(-th, xv[u].x, av[u].x), fma(-th, xv[u].y, av[u].y));
+        if (l < L) r[l] = rv;
+        qr[u] = l < L ? norm2(rv) : 0.f;   // theta may be Inf or NaN
+        qx[u] = norm2(xv[u]);
+      }
+      add_squares(rr, qr);
+      add_squares(xx, qx);
     }
-  }
-  if constexpr (sizeof(T) == 4) {
-    rf.flush(rr);
-    xf.flush(xx);
+  } else {
+    for (size_t l = first; l < L; l += stride) {
+      const cx<T> xv = x[l], av = ax[l];
+      const cx<T> rv = mk(fma(-th, xv.x, av.x), fma(-th, xv.y, av.y));
+      r[l] = rv;
+      if constexpr (sizeof(T) == 4) {
+        rr += (double)norm2(rv);
+        xx += (double)norm2(xv);
+      } else {
+        rr = fma(rv.x, rv.x, fma(rv.y, rv.y, rr));
+        xx = fma(xv.x, xv.x, fma(xv.y, xv.y, xx));
+      }
+    }
   }
   __shared__ double red[2][32];
   for (int o = 16; o > 0; o >>= 1) {
@@ -573,7 +583,7 @@ bool pair_ok(const void* S, const void* Y, size_t L) {
 }
 
 // CTAs per column of the residual kernels: eight entries a thread where the
-// columns are short (each CTA ends with four FP64 atomics on its column's
+// columns are short (each CTA ends with two FP64 atomics on its column's
 // norms; one entry a thread at 32^3 made 384 CTAs of them per column: 16
 // complex128 columns 53 -> 27 us, 16 of 64^3 181 -> 163)
 unsigned residual_grid(size_t L, int nvec) {
@@ -687,12 +697,15 @@ cudaError_t launch_residual(const void* X, const void* AX, const double* theta, 
   cudaError_t e = cudaMemsetAsync(norms, 0, sizeof(double) * 2 * nvec, s);
   if (e != cudaSuccess || nvec == 0) return e;
   dim3 grid(std::max(1u, residual_grid(L, nvec)), nvec);
-  if (precision == PCX_FP64)
-    residual_kernel<double><<<grid, 256, 0, s>>>(static_cast<const cx<double>*>(X), static_cast<const cx<double>*>(AX),
-                                                 theta, static_cast<cx<double>*>(R), norms, nvec, L);
-  else
-    residual_kernel<float><<<grid, 256, 0, s>>>(static_cast<const cx<float>*>(X), static_cast<const cx<float>*>(AX),
-                                                theta, static_cast<cx<float>*>(R), norms, nvec, L);
+  if (precision == PCX_FP64) {
+    residual_kernel<double, false><<<grid, 256, 0, s>>>(static_cast<const cx<double>*>(X),
+                                                        static_cast<const cx<double>*>(AX), theta,
+                                                        static_cast<cx<double>*>(R), norms, nvec, L);
+  } else {
+    const auto kern = L >= (size_t)8 * 256 * grid.x ? residual_kernel<float, true> : residual_kernel<float, false>;
+    kern<<<grid, 256, 0, s>>>(static_cast<const cx<float>*>(X), static_cast<const cx<float>*>(AX), theta,
+                              static_cast<cx<float>*>(R), norms, nvec, L);
+  }
   return cudaGetLastError();
 }
 
