@@ -70,10 +70,10 @@ struct DF {
 };
 
 // Two accumulators in packed pairs: (s, c) += (xh + xl) (yh + yl) in 11 packed
-// operations.  s + c follows Knuth's TwoSum of s and p = fl(xh yh); its terms
-// nb = s_old - s_new and s_old - (s_new + nb) are exact, and the residual of
-// the product and that of the sum, (p + nb) + (xh yh - p), come from one FMA,
-// xh yh + nb.  The product is formed by scalar
+// operations.  s + c follows Knuth's TwoSum of s and p = fl(xh yh): with nb =
+// fl(s_old - s_new) the error of the sum is (s_old - (s_new + nb)) + (p + nb),
+// both terms exact (nb itself need not be).  The second one and the residual of
+// the product, (p + nb) + (xh yh - p), come from one FMA, xh yh + nb.  The product is formed by scalar
 // __fmul_rn: a packed one was fused with the addition that follows it, and
 // TwoSum is exact only for an operand that has been rounded.
 __device__ __forceinline__ void mac_pair(float2& s, float2& c, float2 xh, float2 xl, float2 yh, float2 yl) {

@@ -1,6 +1,6 @@
 // Launchers of the compensated-operator apply (kernels in fft_kernels.cuh,
-// instantiated per precision in fft_f32.cu / fft_f64.cu): vector chunking
-// sized to L2, the context-owned scratch, the file-scope scratch of
+// instantiated per precision in fft_f32.cu / fft_f64.cu): vectors per launch,
+// the context-owned scratch, the file-scope scratch of
 // pcx_apply_noalloc, and the preconditioner launch.
 #include <cuda_runtime.h>
 
@@ -58,7 +58,7 @@ cudaError_t dispatch_apply(const pcx_ctx* c, const KParams& kp, const void* X, v
 // every value 9 times (128^3, four vectors one by one 697 us, in one launch 736;
 // 64^3, 24 vectors in launches of 8 478 us, in one 491); that of complex128,
 // bound by the FP64 pipe, gains by groups (64^3, 24 vectors 3.34 ms in launches
-// of 12, 3.92 in launches of 5).  A context whose scratch could not be allocated
+// of 12, 3.69 in launches of 4).  A context whose scratch could not be allocated
 // stays with what half of L2 holds.
 int apply_chunk(const pcx_ctx* c, int precision) {
   if (c->apply_chunk > 0) return c->apply_chunk;

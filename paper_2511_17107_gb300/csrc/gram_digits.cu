@@ -44,10 +44,11 @@
 // Raw rows arrive by cp.async two chunks ahead, in slots private to the
 // thread that cuts them.
 //
-// What bounds it at 48 x 48: the multiplying warps (mma.sync peaks at 1,036
-// multiply-adds per clock and SM, measured; the kernel reaches half of it,
-// the rest is the addition of the chunk sums, 20 FP32 operations each); narrow
-// products are bound by the cutting warps.  Measured at 3 128^3 rows (GB300):
+// What bounds it at 48 x 48: issue slots and latency of 16 warps (counters at 3 64^3
+// rows: tensor pipe 41%, no pipe above, SM throughput 58%; mma.sync peaks at 1,036
+// multiply-adds per clock and SM, measured); beside the products the multiplying
+// warps add the chunk sums, 20 FP32 operations each.  Narrow products wait for the
+// cutting warps (16 x 16: tensor pipe 20%, FP64 pipe 45%).  Measured at 3 128^3 rows (GB300):
 // complex128 48 x 48 30.4 ms in double-float on the FP32 pipes, 7.2 ms here;
 // 16 x 16 3.46 and 1.58 ms; complex128 x complex64 16 x 32 4.93 and 2.21 ms.
 // (64-bit integer sums of one unit per column, with one conversion per digit

@@ -191,8 +191,8 @@ bool gram_tc_supported(int na, int nb, size_t L);
 bool gram_cc_supported(const void* A, const void* B, int na, int nb, size_t L);
 cudaError_t launch_gram_cc(const void* A, int na, const void* B, int nb, size_t L, double* G, cudaStream_t s);
 void set_gram_path(int path);
-// G = A^H B by integer digits on the tensor cores (gram_digits.cu): prec_a,
-// prec_b the precisions of the column blocks, A complex128
+// G = A^H B by integer digits on the tensor cores (gram_digits.cu): A complex128,
+// prec_b the precision of B
 cudaError_t launch_gram_digits(const void* A, int na, const void* B, int prec_b, int nb, size_t L, double* G,
                                cudaStream_t s);
 void gram_digits_release_stream(cudaStream_t s);

@@ -439,7 +439,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
 // AX = Op X are held and updated in FP64, so the residual R = AX - X Theta
 // is FP64-accurate; the search directions W = K_P^{-1} R, P and their images
 // are FP32 with FP32 applies.  The Rayleigh-Ritz matrices take their X rows
-// from double-float products of the FP64 X, AX with the FP32 directions
+// from digit products of the FP64 X, AX with the FP32 directions
 // (launch_gram_digits), their P/W blocks from tensor-core FP32 products, and their
 // X-X blocks from the previous step (Theta, I).  [P W] is orthonormalised
 // against X in FP32 each step.  An error in a direction block enters the new
@@ -581,8 +581,8 @@ pcx_status lobpcg_refine(Run& r64, Run& r32, int nev, double tol, int maxit, int
     CK(r32.apply(r32.col(r32.S, n), r32.col(r32.AS, n), np + na));
     const int m = n + np + na;
     const int mp = m - n;
-    // Rows of X: X^H [P W] from the FP64 X against the FP32 directions with
-    // double-float sums (these couplings are of the size of the residual, far
+    // Rows of X: X^H [P W] from the FP64 X against the FP32 directions, digit
+    // products (these couplings are of the size of the residual, far
     // below the FP32 rounding of the products), and
     //   (AX)^H [P W] = Theta X^H [P W] + R^H [P W],  R = AX - X Theta,
     // the last term an FP32 product of the rounded FP64 residual (its entries
