@@ -271,20 +271,23 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
   double lrn_best = INFINITY;
   int no_drop = 0;
   res.assign(n, INFINITY);
-  // The eigenvalues of an FP64 run are the Rayleigh quotients x^H AX / x^H x
-  // of the block it returns, off by |residual|^2 / gap.  The Ritz values that
-  // the last step took from an ill-conditioned [X P W] carry the rounding of
-  // its Gram matrices divided by their smallest eigenvalue: up to 1e-9
-  // relative with 10th-order stencils, and the image AX that the steps carry
-  // along adds its own.  One apply and one n x n product per solve.
-  auto quotients = [&](const std::vector<double>& nrm) -> pcx_status {
+  // The eigenvalues of an FP64 run are the Ritz values of the block it returns
+  // alone, from a fresh image: off by |residual|^2 / gap.  Those that the last
+  // step took from an ill-conditioned [X P W] carry the rounding of its Gram
+  // matrices divided by their smallest eigenvalue, up to 1e-9 relative with
+  // 10th-order stencils, and the image AX that the steps carry along adds its
+  // own.  (Quotients of single vectors would mix the values of a cluster.)
+  // One apply and two n x n products per solve.
+  auto block_values = [&]() -> pcx_status {
     if (run.prec != PCX_FP64) return PCX_OK;
     CK(run.apply(run.S.p, run.AS.p, n));
-    std::vector<cd> g;
-    pcx_status s2 = run.gram(run.S.p, n, run.AS.p, n, g);
-    if (s2 != PCX_OK) return s2;
-    for (int j = 0; j < n; ++j) theta[j] = g[(size_t)j * n + j].real() / nrm[n + j];
-    std::sort(theta.begin(), theta.end());
+    std::vector<cd> ga, gb, cm;
+    std::vector<double> th;
+    pcx_status s2;
+    if ((s2 = run.gram(run.S.p, n, run.AS.p, n, ga)) != PCX_OK) return s2;
+    if ((s2 = run.gram(run.S.p, n, run.S.p, n, gb)) != PCX_OK) return s2;
+    if (gen_eig(n, ga, gb, 1e-14, th, cm) == n) theta.assign(th.begin(), th.begin() + n);
+    run.tick(&Times::rr);
     return PCX_OK;
   };
   for (iters = 0;; ++iters) {
@@ -309,7 +312,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
       std::fprintf(stderr, "[pcx] %s it %d worst %.3e theta0 %.12g theta_top %.4e\n",
                    run.prec == PCX_FP64 ? "fp64" : "fp32", iters, worst, theta[0], run.theta_top);
     }
-    if (worst <= tol) return quotients(nrm);
+    if (worst <= tol) return block_values();
     if (worst <= stop_tol) {
       stopped_early = true;
       return PCX_OK;
@@ -329,7 +332,7 @@ pcx_status lobpcg(Run& run, int nev, double tol, int maxit, double stop_tol, int
       stopped_early = true;
       return PCX_OK;
     }
-    if (iters >= maxit) return (st = quotients(nrm)) != PCX_OK ? st : PCX_ENOCONV;
+    if (iters >= maxit) return (st = block_values()) != PCX_OK ? st : PCX_ENOCONV;
     Learned* lrn = run.learned;
     // learned correction: back to the base preconditioner once the worst
     // residual has not dropped 10% below its best for `patience` iterations
