@@ -759,8 +759,9 @@ typedef struct {
  * W = K_P^{-1} R, converged columns keep their place in X but get no new W
  * or P.  Converged when every Res_j <= tol (eq. exp_relativeresidual).  At
  * k = 0 the p = 0 mode of every block is deflated (Prop. 2.5: null space H).
- * Outputs (host, any may be NULL): eig_out[nk*nev] ascending per k,
- * res_out[nk*nev], iters_out[nk].  vec_out: optional DEVICE buffer for the
+ * Outputs (host, any may be NULL): eig_out[nk*nev] ascending per k (the Ritz
+ * values of the final block, its image formed anew), res_out[nk*nev],
+ * iters_out[nk].  vec_out: optional DEVICE buffer for the
  * eigenvectors (nk*nev vectors, FP64 layout).  Synchronises `stream`.
  * Errors: PCX_ENOCONV (cap reached; outputs hold the last iterate),
  * PCX_ENUMERIC (NaN/Inf or unrecoverable breakdown), PCX_EINVAL, PCX_ENOMEM,
